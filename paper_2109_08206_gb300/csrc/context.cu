@@ -106,7 +106,7 @@ void free_all(aLENS_ctx* c)
     void* ptrs[] = {c->xw, c->axis, c->unc, c->pos32, c->ax32, c->cellkey, c->sorted_id, c->spos32, c->sax32,
                     c->cell_count, c->cell_start, c->cell_cursor, c->rod_count, c->rod_ncand, c->rod_tmpstart, c->cand,
                     c->rowP, c->rowQ, c->cntQ, c->curQ, c->qlist, c->perm, c->rank, c->curP, c->ci, c->cj, c->pairs, c->phi, c->dgeom,
-                    c->q64, c->scale64, c->solve_ws, c->partials, c->bstart, c->bar, c->dflags, c->dcount, c->scan_tmp,
+                    c->q64, c->scale64, c->solve_ws, c->partials, c->xch, c->bstart, c->bar, c->dflags, c->dcount, c->scan_tmp,
                     c->systab, c->sysid, c->sysoff, c->sys_order, c->sys_iters, c->sys_res, c->adj_ws,
                     c->sp_ends, c->sp_arms, c->sp_kappa, c->sp_rest, c->comp64, c->fnc_buf, c->gin_buf,
                     c->row_keys, c->prev_keys, c->prev_gam};
@@ -426,9 +426,10 @@ aLENS_status aLENS_create(const aLENS_params* params, int64_t max_rods, int64_t 
     ok &= dmalloc(&c->scale64, mp * sizeof(double)) == cudaSuccess;
     // solver buffers, sized for float64; the float32 views alias the same memory
     // every slice starts on a 64-byte boundary (vector loads): 8 elements of slack each
-    size_t solve_elems = 9 * mp + 8 * mp + mp + 3 * np + 8 * mp + 18 * np + mp + 4 * np + mp + mp + 8 * 14 + 8 * mp;
+    size_t solve_elems = 9 * mp + 8 * mp + mp + 3 * np + 8 * mp + 12 * np + mp + 4 * np + mp + mp + 8 * 14 + 8 * mp;
     ok &= dmalloc((char**)&c->solve_ws, solve_elems * sizeof(double)) == cudaSuccess;
     ok &= dmalloc(&c->partials, ((size_t)c->max_blocks + 4) * 8 * sizeof(double)) == cudaSuccess;
+    ok &= dmalloc(&c->xch, xch_bytes(np, (size_t)c->max_blocks)) == cudaSuccess;
     ok &= dmalloc(&c->bstart, ((size_t)c->max_blocks + 1) * sizeof(int)) == cudaSuccess;
     ok &= dmalloc(&c->bar, 4 * sizeof(unsigned)) == cudaSuccess;
     ok &= dmalloc(&c->dflags, F_NFLAGS * sizeof(int)) == cudaSuccess;
@@ -452,13 +453,15 @@ aLENS_status aLENS_create(const aLENS_params* params, int64_t max_rods, int64_t 
         size_t o = 0;
         auto carve64 = [&](size_t cnt) { double* r = base + o; o = (o + cnt + 7) & ~(size_t)7; return r; };
         SolveBufs<double>& s = c->sb64;
-        s.gg[0] = carve64(4 * mp); s.gg[1] = carve64(4 * mp); s.U = carve64(6 * np); s.U2 = carve64(6 * np);
+        s.gg[0] = carve64(4 * mp); s.gg[1] = carve64(4 * mp); s.U = carve64(6 * np);
         s.Uref = carve64(6 * np);
         s.gref = carve64(mp);
         s.rec = carve64(9 * mp); s.qe = carve64(8 * mp); s.q = carve64(mp); s.ax = carve64(3 * np);
         s.mobr = carve64(4 * np);
         s.comp = carve64(mp);
         s.isc = carve64(mp);
+        s.priv = s.qe;
+        s.hrank = (int*)(s.qe + 2 * mp);
         s.pe = nullptr;   // the float64 rod phase reads rec (its arithmetic bounds it)
         s.lop = nullptr;
         s.loq = nullptr;
@@ -466,16 +469,18 @@ aLENS_status aLENS_create(const aLENS_params* params, int64_t max_rods, int64_t 
         size_t f = 0;
         auto carve32 = [&](size_t cnt) { float* r = fb + f; f = (f + cnt + 7) & ~(size_t)7; return r; };
         SolveBufs<float>& t = c->sb32;
-        t.gg[0] = carve32(4 * mp); t.gg[1] = carve32(4 * mp); t.U = carve32(6 * np); t.U2 = carve32(6 * np);
+        t.gg[0] = carve32(4 * mp); t.gg[1] = carve32(4 * mp); t.U = carve32(6 * np);
         t.Uref = carve32(6 * np);
         t.gref = carve32(mp);
         t.rec = carve32(9 * mp); t.qe = carve32(8 * mp); t.q = carve32(mp); t.ax = carve32(3 * np);
+        t.priv = t.qe;
+        t.hrank = (int*)(t.qe + 2 * mp);
         t.mobr = carve32(4 * np);
         t.comp = carve32(mp);
         t.isc = carve32(mp);
         t.pe = carve32(8 * mp);
-        // the float32 views use at most 71 mp + 25 np of the workspace's
-        // 74 mp + 50 np floats: room for the owner-side records, the low
+        // the float32 views use at most 71 mp + 19 np of the workspace's
+        // 74 mp + 38 np floats: room for the owner-side records, the low
         // parts and their rows
         t.rec_lo = carve32(9 * mp); t.qe_lo = carve32(8 * mp); t.q_lo = carve32(mp);
         t.lop = carve32(8 * mp); t.loq = carve32(8 * mp);

@@ -40,6 +40,15 @@ inline size_t sys_queue_ints(int ns) { return (size_t)ns + 2 * ((size_t)ns + kMa
 enum Count : int { C_PAIRS = 0, C_OVERLAP = 1, C_MINGAP = 2, C_CAND = 3, C_RESID = 4, C_ALPHA0 = 5, C_SMEM = 6,
                    C_QUEUE = 7, C_WALLS = 8, C_MAXRODS = 9, C_SMEM1 = 10, C_MEFF = 11, C_NCOUNT = 12 };
 
+// The one-barrier solver's exchange area (16-byte tagged words): two
+// velocity buffers of at most kXchRodWords words a rod, then kSumSlots sets of
+// block sums, kSumWords words a block.
+constexpr int kXchRodWords = 4, kSumSlots = 4, kSumWords = 4;
+constexpr size_t xch_bytes(size_t rods, size_t blocks)
+{
+    return 16 * (2 * kXchRodWords * rods + (size_t)kSumSlots * kSumWords * blocks);
+}
+
 // Constraint count of a launch: m itself, or, for a step that runs without
 // host readbacks (a captured graph: grids sized for the capacity m), the
 // count the device holds in *mdev, at most m.
@@ -283,7 +292,6 @@ struct SolveBufs {           // typed views into the solver workspace
     T* ax;                   // [3][np]
     T* gg[2];                // [mp][4] x 2: (delta, g, gamma_ref, 0), ping-pong
     T* U;                    // [np][6] velocity increment M D delta
-    T* U2;                   // [np][6] second increment buffer (the one-barrier solver alternates U, U2)
     T* Uref;                 // [np][6] reference velocity M D gamma_ref
     T* gref;                 // [mp] reference gradient q + D^T Uref
     T* mobr;                 // [4][np] per-rod inverse drags (batches)
@@ -294,6 +302,8 @@ struct SolveBufs {           // typed views into the solver workspace
     T* q_lo;                 // [mp]
     T* lop;                  // [mp][8] rec_lo of the owner side (e, y_P x e, 2 pad) as one row
     T* loq;                  // [mp][8] rec_lo of the other side (e, y_Q x e, 2 pad) (null: read rec_lo)
+    T* priv;                 // [2][mp] the one-barrier solver's spill (qe's space, which it does not read)
+    int* hrank;              // [2 mp] its blocks' halo ranks (the two-barrier kernels' space as well)
     T* comp;                 // [mp] < 0 collision, >= 0 spring compliance 1/(h kappa) (solver order)
     T* isc;                  // [mp] 1 / sigma_c: the constraint's scaling undone (solver order)
 };
@@ -347,7 +357,8 @@ struct aLENS_ctx {
     void* solve_ws;          // typed solver buffers (sized for double)
     alens::SolveBufs<double> sb64;
     alens::SolveBufs<float> sb32;
-    double* partials;        // [max_blocks + 4][8]: [4][nb] block sums, or [2][4][nb] (one-barrier solver)
+    double* partials;        // [max_blocks + 4][8]: [4][nb] block sums
+    uint4* xch;              // one-barrier solver's tagged words: 2 velocity buffers (at most 4 words a rod), block sums
     int max_blocks;
     int* bstart;             // [max_blocks + 1] solver block boundaries (rod ranks)
     unsigned* bar;           // [4]

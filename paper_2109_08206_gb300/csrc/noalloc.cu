@@ -53,6 +53,16 @@ constexpr size_t kNoallocScratchBytes =
 // the header states the size as 5.19 MB
 static_assert(kNoallocScratchBytes > 5180000 && kNoallocScratchBytes < 5195000, "noalloc scratch size changed");
 
+// The one-barrier solver's exchange words (float32 ones take half of
+// kXchRodWords a rod) and spill, both in the space of qe.  At most 32 rods a
+// block up to one block per SM.
+constexpr int kNoallocBlocks1 = (kNoallocMaxRods + 31) / 32;
+constexpr size_t kXch32 = xch_bytes(kNoallocMaxRods / 2, kNoallocBlocks1);
+constexpr size_t kXch64 = xch_bytes(kNoallocMaxRods, kNoallocBlocks1);
+static_assert(kXch32 + 2 * sizeof(float) * (size_t)kNoallocMaxPairs <= 8 * sizeof(float) * (size_t)kNoallocMaxPairs &&
+                  kXch64 + 3 * sizeof(double) * (size_t)kNoallocMaxPairs <= 8 * sizeof(double) * (size_t)kNoallocMaxPairs,
+              "the exchange area and the spill do not fit qe");
+
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
 std::mutex g_lock;
@@ -149,7 +159,7 @@ extern "C" aLENS_status aLENS_solve_lcp_noalloc(const aLENS_params* params, int6
         double* b64 = (double*)c.solve_ws;
         size_t u = 0;
         auto c64 = [&](size_t cnt) { double* r = b64 + u; u = (u + cnt + 7) & ~(size_t)7; return r; };
-        c.sb64.gg[0] = c64(4 * mp); c.sb64.gg[1] = c64(4 * mp); c.sb64.U = c64(6 * np); c.sb64.U2 = c64(6 * np);
+        c.sb64.gg[0] = c64(4 * mp); c.sb64.gg[1] = c64(4 * mp); c.sb64.U = c64(6 * np);
         c.sb64.Uref = c64(6 * np);
         c.sb64.gref = c64(mp);
         c.sb64.rec = c64(9 * mp); c.sb64.qe = c64(8 * mp); c.sb64.q = c64(mp); c.sb64.ax = c64(3 * np);
@@ -159,7 +169,7 @@ extern "C" aLENS_status aLENS_solve_lcp_noalloc(const aLENS_params* params, int6
         float* b32 = (float*)c.solve_ws;
         size_t v = 0;
         auto c32 = [&](size_t cnt) { float* r = b32 + v; v = (v + cnt + 7) & ~(size_t)7; return r; };
-        c.sb32.gg[0] = c32(4 * mp); c.sb32.gg[1] = c32(4 * mp); c.sb32.U = c32(6 * np); c.sb32.U2 = c32(6 * np);
+        c.sb32.gg[0] = c32(4 * mp); c.sb32.gg[1] = c32(4 * mp); c.sb32.U = c32(6 * np);
         c.sb32.Uref = c32(6 * np);
         c.sb32.gref = c32(mp);
         c.sb32.rec = c32(9 * mp); c.sb32.qe = c32(8 * mp); c.sb32.q = c32(mp); c.sb32.ax = c32(3 * np);
@@ -167,7 +177,17 @@ extern "C" aLENS_status aLENS_solve_lcp_noalloc(const aLENS_params* params, int6
         c.sb32.comp = c32(mp);
         c.sb32.isc = c32(mp);
         // the float32 views use at most half of the workspace: room for the low parts
+        // the one-barrier solver's exchange words and its spill take the place of qe, which it does not read
+        if (params->precision == ALENS_MIXED) {
+            c.xch = reinterpret_cast<uint4*>(c.sb32.qe);
+            c.sb32.priv = c.sb32.qe + kXch32 / sizeof(float);
+        } else {
+            c.xch = reinterpret_cast<uint4*>(c.sb64.qe);
+            c.sb64.priv = c.sb64.qe + kXch64 / sizeof(double);
+            c.sb64.hrank = reinterpret_cast<int*>(c.sb64.priv + 2 * mp);
+        }
         c.sb32.rec_lo = c32(9 * mp); c.sb32.qe_lo = c32(8 * mp); c.sb32.q_lo = c32(mp);
+        c.sb32.hrank = reinterpret_cast<int*>(c.sb32.qe_lo);   // (as qe)
     }
 
     int hflags[F_NFLAGS];

@@ -154,13 +154,19 @@ __device__ __forceinline__ void st_ref(T* p, int c, T gr, T gl)
     reinterpret_cast<typename V2<T>::t*>(p)[2 * (size_t)c + 1] = v;
 }
 
+// Sums that are never fused with a product they add (the compiler may
+// otherwise take a + (rounded p q) as fma(p, q, a), as it likes in each
+// place, which breaks the error-free transformations below).
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
 // Exact sum: a + b = s + e.
 template <typename T>
 __device__ __forceinline__ void two_sum(T a, T b, T& s, T& e)
 {
-    s = a + b;
-    const T bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
+    s = add_rn(a, b);
+    const T bb = add_rn(s, -a);
+    e = add_rn(add_rn(a, -add_rn(s, -bb)), add_rn(b, -bb));
 }
 
 // Sum-of-products accumulator.  COMP (float32 reference passes): an
@@ -205,9 +211,13 @@ struct SolveArgs {
     T* gg0;     // [m][4] (delta, g, gamma_ref, 0): written inside the kernel, plain (coherent) loads only
     T* gg1;
     T* U;       // [n][6] velocity increment M D delta
-    T* U2;      // [n][6] second increment buffer (one-barrier solver)
     T* Uref;    // [n][6] reference velocity M D gamma_ref
     T* gref;    // [m] reference gradient q + D^T Uref (blocks working from global memory)
+    T* priv;       // one-barrier solver: 2 mp values for what a share's shared memory does not hold (qe's space)
+    int* hrank;    // one-barrier solver: ranks of the blocks' halo rods (2 mp)
+    size_t dyn_bytes;   // its dynamic shared memory
+    uint4* xch;    // one-barrier solver: tagged velocities [2][n] rods, then tagged block sums [kSumSlots][blocks]
+    int workers;   // one-barrier solver: threads that hold slots and rods (a further warp, if any, sums the blocks)
     double* partials;
     unsigned* bar;
     int* flags;
@@ -1157,7 +1167,7 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd(SolveArgs<T> a)
 }
 
 // ---------------------------------------------------------------------
-// One grid barrier per iteration (staged blocks).
+// No grid barrier in an iteration (staged blocks).
 //
 // The loop above exchanges two things between blocks in every iteration:
 // the velocities dU, which the constraint phase gathers, and the state of
@@ -1169,56 +1179,108 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd(SolveArgs<T> a)
 // (the same delta, g and alpha, the same two velocities, the same order of
 // operations), so that owner and ghost stay equal bit for bit and the rod
 // phase reads nothing but shared memory.  Only dU and the block sums cross
-// blocks, and both travel on one barrier:
+// blocks, and both travel as tagged words (below), so that no iteration
+// waits on a grid barrier:
 //   constraint phase k (every owned and ghost constraint):
-//       delta_k = max(-gamma_ref, delta_{k-1} - alpha_{k-1} g_{k-1}),
-//       g_k = gref + D^T dU_k, and for owned constraints the sums of
-//       s.s, s.y, y.y (s = delta_k - delta_{k-1}, y = g_k - g_{k-1}) and
-//       max |pi_k|;
-//   step decision from the sums of constraint phase k-1 (published by the
-//       last barrier, fetched into shared memory by cp.async while the
-//       constraint phase runs): alpha_k = BB(s_{k-2}, y_{k-2}), i.e. the
-//       Barzilai-Borwein step of the published method taken one iteration
-//       late (a gradient method with retards: Friedlander, Martinez, Molina
-//       & Raydan, SIAM J. Numer. Anal. 36, 1999);
-//   rod phase k: delta_{k+1} formed on the fly, dU_{k+1} = M D delta_{k+1},
-//       copied out to one of two global buffers (they alternate, so a block
-//       never overwrites velocities another block may still be reading);
-//   grid barrier (block sums in one of two buffers, alternating alike).
+//       g_k = gref + D^T dU_k, for owned constraints the sums of s.s, s.y,
+//       y.y (s = delta_k - delta_{k-1}, y = g_k - g_{k-1}) and max |pi_k|,
+//       and delta_{k+1} = max(-gamma_ref, delta_k - alpha_k g_k);
+//   rod phase k: dU_{k+1} = M D delta_{k+1}, published rod by rod;
+//   step decision, by a warp of its own while the others run the rod phase,
+//       from the sums of constraint phase k: alpha_{k+1} =
+//       BB(s_{k-1}, y_{k-1}), i.e. the Barzilai-Borwein step of the
+//       published method taken one iteration late (a gradient method with
+//       retards: Friedlander, Martinez, Molina & Raydan, SIAM J. Numer.
+//       Anal. 36, 1999), which leaves the sums the rod phase to arrive in.
 // A residual below tol, 64 float32 iterations, or max_iter start a
 // reference refresh of the iterate the slots hold (the same compensated
-// passes as above, two extra barriers); the loop stops only on the residual
-// of a fresh reference, so the returned gamma (delta = 0 there) carries the
-// residual it reports, in float64 and float32 alike.
+// passes as above, with one grid barrier); the loop stops only on the
+// residual of a fresh reference, so the returned gamma (delta = 0 there)
+// carries the residual it reports, in float64 and float32 alike.
+//
+// Tagged words: 12 bytes of values and a 32-bit exchange number in one
+// 16-byte word, stored and loaded whole (ld/st .b128, relaxed).  A reader
+// polls the word it needs until its number is the iteration's, so a
+// velocity costs one store and one load across L2, where a grid barrier
+// costs the fence over the block's stores, the arrival, the poll and then
+// the load.  A word is rewritten two exchanges (velocities) or kSumSlots
+// exchanges (sums) later: a block writes dU_{k+2} after decision k+1, which
+// took every block's sums of constraint phase k, and a block publishes those
+// once all its threads have read dU_k; likewise it publishes sums k + 2
+// after decision k + 2, which took every block's sums k + 1, and a block
+// publishes those after decision k + 1, when it has read all the sums k.
+//
+// What bounds it: two messages across L2 an iteration (velocities, sums; one
+// way 700-1080 cycles, all blocks' words at every block about 2500) and the
+// latency of the two phases; the data sit in shared memory.  Solve times
+// before (one grid barrier an iteration) and after, the same bits: 1e3 rods
+// float64 5.09 -> 2.01 ms (219 iterations), 1e3 rods with walls 0.71 -> 0.43
+// ms a step, 5e3 rods 0.86 -> 0.66, 2e4 rods 1.98 -> 1.45, 5e4 rods 1.43 ->
+// 1.25, 1e5 rods 3.90 -> 3.60 (366 iterations), 1e4 rods float64 2.17 -> 1.56.
+// Where the rods come in no spatial order (a large solve_lcp) nearly every
+// slot's other end is in the halo and the polls cost more than they save: 5e4
+// rods 2.08 -> 2.50.
 
 // A block's share: rods [r0, r1), owned constraints [c0, c1) in slots
 // [0, nc), ghosts in slots [nc, nt).
+//
+// A slot is three rows of four values, so that one rod's entry is two
+// 16-byte loads of shared memory (float32) instead of eight 4-byte gathers:
+//   row 0  e_x e_y e_z, the increment delta
+//   row 1  y_P x e,     gamma_ref
+//   row 2  y_Q x e,     gref = q + D^T Uref (gamma_lo during a refresh)
+// Slot nt is all zero.  The constraint phase leaves delta_{k+1}, the rod
+// phase's input, in row 0.  A rod's entries, owned then other-side, are
+// 16-bit slot numbers (kOther: the rod is the slot's Q side), padded to a
+// multiple of four with the zero slot, so that four come in one load and the
+// loop has no tail.
+//
+// Velocities are rows too: the block's rods, one zero row (the other end of a
+// wall contact) and the halo, every rod of another block that a slot touches,
+// fetched once per iteration however many slots read it.  A slot knows the rows
+// of its P and Q ends.
+//
+// The share's description lives in shared memory, its arrays as offsets into
+// the block's dynamic shared memory: held in registers it pushed the kernel
+// past the 72 a thread has, and what spilled went to L2, since shared memory
+// leaves little L1.
+template <typename X>
+__device__ __forceinline__ X* smem_at(int off)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    return reinterpret_cast<X*>(dyn + off);
+}
 template <typename T>
 struct Own1 {
-    int r0, r1, c0, c1, q0, q1, nc, ng, nt, cap_r, nbp;
-    T* tot;      // [4][nbp] last barrier's block sums (cp.async target)
-    T* rec;      // [9][nt]
-    T* gref;     // [nt] q + D^T Uref
-    T* ds;       // [nt] delta
-    T* grs;      // [nt] g
-    T* gam;      // [nt] gamma_ref
-    T* ax;       // [3][cap_r]
-    T* U;        // [6][cap_r] this iteration's dU (the reference velocity during a refresh)
-    int* oth;    // [nt] rank of the slot's other end: Q for owned slots, the owner for ghosts (-1: a wall)
-    int* gid;    // [ng] constraint id of ghost slot nc + g
-    int* rowP;   // [cap_r + 1] owned ranges (constraint ids; slot = id - c0)
-    int* rowQ;   // [cap_r + 1] other-side ranges (CSR positions)
-    unsigned short* loc;    // [nt] local index of the slot's rod in this block (P owned, Q ghost), | kBil
-    unsigned short* qslot;  // [q1 - q0] slot of each other-side entry, | kBil
-    unsigned short* perm;   // [cap_r] rod order of the rod phase
+    int r0, r1, c0, c1, q0, q1, nc, ng, nt, cap_r;
+    int ne;      // entries, padding included
+    int nh;      // halo rods
+    int halo;    // their rows fit (else every slot polls for itself)
+    T* ds;       // [nc] delta before the last step (owned slots: the step's s)
+    T* gs;       // [nc] g of the last step (owned slots: the step's y)
+    int* gid;    // [ng] constraint id of ghost slot nc + g (global memory)
+    int* hrank;  // [nh] rank of each halo rod (global memory)
+    int off_ax, off_ij, off_ent, off_rowE, off_perm, off_U;
+    using u16 = unsigned short;
+    __device__ __forceinline__ T* row() const { return smem_at<T>(0); }             // [3][nt + 1][4]
+    __device__ __forceinline__ T* ax() const { return smem_at<T>(off_ax); }         // [3][cap_r]
+    __device__ __forceinline__ T* U() const { return smem_at<T>(off_U); }           // [cap_r + 1 + nh][6] this iteration's dU (Uref in a refresh)
+    __device__ __forceinline__ unsigned* ij() const { return smem_at<unsigned>(off_ij); }   // [nt] velocity rows of P (low half) and Q
+    __device__ __forceinline__ u16* ent() const { return smem_at<u16>(off_ent); }   // [ne]
+    __device__ __forceinline__ u16* rowE() const { return smem_at<u16>(off_rowE); } // [cap_r + 1] first entry of each rod, in fours
+    __device__ __forceinline__ u16* perm() const { return smem_at<u16>(off_perm); } // [cap_r] rod order of the rod phase
 };
-constexpr unsigned kBil = 0x8000u;   // bilateral (spring) constraint: no projection
-constexpr int kMaxSlots = 0x7fff;
+constexpr unsigned kOther = 0x8000u;
+constexpr int kMaxSlots = 0x7ffe;
 
 __host__ __device__ inline size_t align16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-// Shared-memory bytes of a one-barrier block share (nt slots of which ng
-// ghosts, nr rods, nq other-side entries, nb blocks).
+// Whether a share (nt slots of which ng ghosts, nr rods, nq other-side
+// entries, nb blocks) is the one-barrier kernel's: 13 values a slot, 9 a rod
+// and the indices within the shared-memory budget.  The bound decides which
+// kernel solves a system, and with it every bit of the result, so it stays
+// where it was drawn; carve1 needs about as much (and leaves ds and gs to
+// global memory where a share would not fit).
 __host__ __device__ inline size_t staged1_bytes(int esize, size_t nt, size_t ng, size_t nr, size_t nq, size_t nb)
 {
     const size_t nbp = (nb + 3) & ~(size_t)3;
@@ -1226,111 +1288,183 @@ __host__ __device__ inline size_t staged1_bytes(int esize, size_t nt, size_t ng,
            align16((nt + ng + 2 * nr + 2) * sizeof(int)) + align16((nt + nq + nr) * sizeof(unsigned short));
 }
 
+// Carves the share out of the block's dynamic shared memory.  12 (nt + 1) +
+// 9 nr + 6 values, nt words and at most nt + nq + 5 nr + 1 16-bit words are
+// no more than staged1_bytes, so they always fit; the halo and then ds and gs
+// take what is left of cap bytes (carve_rest, once the halo is counted).
 template <typename T>
-__device__ void carve1(Own1<T>& o, unsigned char* base)
+__device__ void carve1(Own1<T>& o)
 {
-    const size_t nt = o.nt, R = o.cap_r;
-    o.tot = reinterpret_cast<T*>(base);
-    base += align16(4 * (size_t)o.nbp * sizeof(T));
-    T* t = reinterpret_cast<T*>(base);
-    o.rec = t; t += 9 * nt;
-    o.gref = t; t += nt;
-    o.ds = t; t += nt;
-    o.grs = t; t += nt;
-    o.gam = t; t += nt;
-    o.ax = t; t += 3 * R;
-    o.U = t; t += 6 * R;
-    base += align16((13 * nt + 9 * R) * sizeof(T));
-    int* ip = reinterpret_cast<int*>(base);
-    o.oth = ip; ip += nt;
-    o.gid = ip; ip += o.ng;
-    o.rowP = ip; ip += R + 1;
-    o.rowQ = ip; ip += R + 1;
-    base += align16((nt + o.ng + 2 * R + 2) * sizeof(int));
-    unsigned short* sp = reinterpret_cast<unsigned short*>(base);
-    o.loc = sp; sp += nt;
-    o.qslot = sp; sp += o.q1 - o.q0;
-    o.perm = sp;
+    const int nt = o.nt, R = o.cap_r;
+    int at = 12 * (nt + 1) * (int)sizeof(T);
+    o.off_ij = at; at += 4 * nt;
+    o.off_ax = (int)(((size_t)at + sizeof(T) - 1) & ~(sizeof(T) - 1)); at = o.off_ax + 3 * R * (int)sizeof(T);
+    o.off_ent = (at + 7) & ~7; at = o.off_ent + 2 * o.ne;   // (fours of entries on 8-byte boundaries)
+    o.off_rowE = at; at += 2 * (R + 1);
+    o.off_perm = at; at += 2 * R;
+    o.off_U = (int)align16((size_t)at);   // (vector loads)
 }
+
+template <typename T>
+__device__ void carve_rest(Own1<T>& o, size_t cap, T* priv, size_t mp)
+{
+    size_t used = o.off_U + 6 * (size_t)(o.cap_r + 1) * sizeof(T);
+    const size_t h = 6 * (size_t)o.nh * sizeof(T), d = 2 * (size_t)o.nc * sizeof(T);
+    o.halo = used + h <= cap;
+    if (o.halo) used += h;
+    if (used + d <= cap) {
+        o.ds = smem_at<T>((int)used);
+        o.gs = o.ds + o.nc;
+    } else {
+        o.ds = priv + o.c0;
+        o.gs = priv + mp + o.c0;
+    }
+}
+
+// ------------------------------------------------- tagged 16-byte words
+__device__ __forceinline__ void st_word(uint4* p, unsigned x, unsigned y, unsigned z, unsigned tag)
+{
+    asm volatile("{\n\t.reg .b64 lo, hi;\n\t.reg .b128 v;\n\tmov.b64 lo, {%1, %2};\n\tmov.b64 hi, {%3, %4};\n\t"
+                 "mov.b128 v, {lo, hi};\n\tst.relaxed.gpu.global.b128 [%0], v;\n\t}"
+                 ::"l"(p), "r"(x), "r"(y), "r"(z), "r"(tag) : "memory");
+}
+__device__ __forceinline__ uint4 ld_word(const uint4* p)
+{
+    uint4 r;
+    asm volatile("{\n\t.reg .b64 lo, hi;\n\t.reg .b128 v;\n\tld.relaxed.gpu.global.b128 v, [%4];\n\t"
+                 "mov.b128 {lo, hi}, v;\n\tmov.b64 {%0, %1}, lo;\n\tmov.b64 {%2, %3}, hi;\n\t}"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p) : "memory");
+    return r;
+}
+
+// K values of T in ceil(K sizeof(T) / 12) tagged words; get returns whether
+// all of them carry the tag.
+template <typename T, int K> struct Tagged;
+template <int K>
+struct Tagged<float, K> {
+    static constexpr int kWords = (K + 2) / 3;
+    static __device__ __forceinline__ void put(uint4* p, const float* v, unsigned tag)
+    {
+#pragma unroll
+        for (int w = 0; w < kWords; ++w)
+            st_word(p + w, __float_as_uint(v[3 * w]), 3 * w + 1 < K ? __float_as_uint(v[3 * w + 1]) : 0u,
+                    3 * w + 2 < K ? __float_as_uint(v[3 * w + 2]) : 0u, tag);
+    }
+    static __device__ __forceinline__ bool get(const uint4* p, unsigned tag, float* v)
+    {
+        uint4 r[kWords];
+        bool ok = true;
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) r[w] = ld_word(p + w);
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) {
+            ok = ok && r[w].w == tag;
+            v[3 * w] = __uint_as_float(r[w].x);
+            if (3 * w + 1 < K) v[3 * w + 1] = __uint_as_float(r[w].y);
+            if (3 * w + 2 < K) v[3 * w + 2] = __uint_as_float(r[w].z);
+        }
+        return ok;
+    }
+};
+template <int K>
+struct Tagged<double, K> {   // two words hold three values
+    static constexpr int kWords = (2 * K + 2) / 3;
+    static __device__ __forceinline__ void put(uint4* p, const double* v, unsigned tag)
+    {
+        unsigned h[3 * kWords] = {};
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(v[k]);
+            h[2 * k] = (unsigned)b;
+            h[2 * k + 1] = (unsigned)(b >> 32);
+        }
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) st_word(p + w, h[3 * w], h[3 * w + 1], h[3 * w + 2], tag);
+    }
+    static __device__ __forceinline__ bool get(const uint4* p, unsigned tag, double* v)
+    {
+        unsigned h[3 * kWords];
+        uint4 r[kWords];
+        bool ok = true;
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) r[w] = ld_word(p + w);
+#pragma unroll
+        for (int w = 0; w < kWords; ++w) {
+            ok = ok && r[w].w == tag;
+            h[3 * w] = r[w].x; h[3 * w + 1] = r[w].y; h[3 * w + 2] = r[w].z;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            v[k] = __longlong_as_double((long long)((unsigned long long)h[2 * k] | (unsigned long long)h[2 * k + 1] << 32));
+        return ok;
+    }
+};
+template <typename T> using Xch = Tagged<T, 6>;      // a rod's velocity
+template <typename T> using XchSum = Tagged<T, 4>;   // a block's sums
+static_assert(Xch<double>::kWords <= kXchRodWords && XchSum<double>::kWords <= kSumWords, "xch_bytes");
+// K values at p, polled until all their words carry the tag.  Bounded like
+// grid_barrier: after wait_cycles, or when any block has recorded an error,
+// it records ALENS_ERR_TIMEOUT, sets *bad and returns what it read last.
+template <typename T, int K>
+__device__ __forceinline__ void get_tagged(int* flags, long long wait_cycles, const uint4* p, unsigned tag, int* bad, T* v)
+{
+    if (Tagged<T, K>::get(p, tag, v)) return;
+    const long long t0 = clock64();
+    for (unsigned polls = 1; !Tagged<T, K>::get(p, tag, v); ++polls) {
+        if ((polls & 15u) == 0) {
+            const bool late = clock64() - t0 > wait_cycles || polls > (1u << 28);
+            if (late) atomicCAS(&flags[F_SOLVE_ERR], 0, ALENS_ERR_TIMEOUT);
+            if (late || ld_volatile_i32(&flags[F_SOLVE_ERR]) != 0) {
+                *(volatile int*)bad = 1;
+                return;
+            }
+        }
+    }
+}
+
+// The slots' and rods' first item of this thread (none for the warp beyond the workers).
+template <typename T>
+__device__ __forceinline__ int first_item(const SolveArgs<T>& a)
+{
+    return (int)threadIdx.x < a.workers ? (int)threadIdx.x : 0x40000000;
+}
+
+// hi > lo ? hi : lo
+template <typename T>
+__device__ __forceinline__ T max_of(T lo, T hi) { return hi > lo ? hi : lo; }
 
 template <typename T>
 struct Shared1 {
-    T red[32][4];
-    T tot[4];   // grid totals of the last barrier's block sums (warps 1-4, one each)
+    Own1<T> o;
+    T red[32][4];           // (sort_rods_total's counters before the first iteration)
     T alpha;
-    int kind, ng;
+    T alpha0, pimax;        // step state, kept by the duty warp's lane 0
+    int k, since, hist;
+    int kind, ng, nh, ne;
+    int nref;               // refreshes taken: the reference lives in state buffer nref & 1
+    unsigned epoch;         // grid barriers passed (thread 0's)
+    int bad;    // a wait ran out (or another block's did): the block leaves
 };
 
-// Stage one slot (owned or ghost) of constraint c from the global arrays.
-template <typename T>
-__device__ __forceinline__ void stage_slot(const SolveArgs<T>& a, const Own1<T>& o, int t, int c, int li, int other,
-                                           unsigned bil)
+template <typename T> struct Row { T x, y, z, w; };
+__device__ __forceinline__ Row<float> ld_row(const float* p)
 {
-    const size_t mp = a.mp, nt = o.nt;
-#pragma unroll
-    for (int w = 0; w < 9; ++w) o.rec[w * nt + t] = a.rec[w * mp + c];
-    T d, g, gr, gl;
-    ld_state(a.gg0, c, d, g, gr, gl);
-    o.ds[t] = d;
-    o.gam[t] = gr;
-    o.grs[t] = gl;   // gamma_lo until the first reference pass replaces it by g
-    o.gref[t] = T(0);
-    o.oth[t] = other;
-    o.loc[t] = (unsigned short)(li | bil);
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    return {v.x, v.y, v.z, v.w};
 }
-
-template <typename T>
-__device__ void stage_in1(const SolveArgs<T>& a, Own1<T>& o, unsigned char* dyn, Shared1<T>& sh)
+__device__ __forceinline__ Row<double> ld_row(const double* p)
 {
-    const int nr = o.r1 - o.r0, nq = o.q1 - o.q0;
-    // ghosts: other-side entries of the block's rods that another block owns
-    if (threadIdx.x == 0) sh.ng = 0;
-    __syncthreads();
-    int cnt = 0;
-    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
-        const int c = a.qlist[o.q0 + k];
-        cnt += c < o.c0 || c >= o.c1;
-    }
-    if (cnt) atomicAdd(&sh.ng, cnt);
-    __syncthreads();
-    o.ng = sh.ng;
-    o.nt = o.nc + o.ng;
-    carve1(o, dyn);
-    __syncthreads();
-    if (threadIdx.x == 0) sh.ng = 0;
-    for (int li = threadIdx.x; li <= nr; li += blockDim.x) {
-        o.rowP[li] = a.rowP[o.r0 + li];
-        o.rowQ[li] = a.rowQ[o.r0 + li];
-    }
-    for (int li = threadIdx.x; li < nr; li += blockDim.x)
-        for (int w = 0; w < 3; ++w) o.ax[w * o.cap_r + li] = a.ax[w * (size_t)a.np + o.r0 + li];
-    const bool has_comp = a.comp != nullptr;
-#pragma unroll 1
-    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) {
-        const int c = o.c0 + t;
-        const unsigned bil = has_comp && a.comp[c] >= T(0) ? kBil : 0u;
-        stage_slot(a, o, t, c, a.ci[c] - o.r0, a.cj[c], bil);
-    }
-    __syncthreads();   // sh.ng is 0 again before the slots are numbered
-#pragma unroll 1
-    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
-        const int c = a.qlist[o.q0 + k];
-        const unsigned bil = has_comp && a.comp[c] >= T(0) ? kBil : 0u;
-        int t;
-        if (c < o.c0 || c >= o.c1) {
-            // the slot order of ghosts does not enter any result
-            const int g = atomicAdd(&sh.ng, 1);
-            t = o.nc + g;
-            o.gid[g] = c;
-            stage_slot(a, o, t, c, a.cj[c] - o.r0, a.ci[c], bil);
-        } else {
-            t = c - o.c0;
-        }
-        o.qslot[k] = (unsigned short)(t | bil);
-    }
-    __syncthreads();
-    sort_rods(o.rowP, o.rowQ, nr, reinterpret_cast<unsigned*>(o.U), reinterpret_cast<int*>(o.U) + nr, o.perm);
+    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+    return {a.x, a.y, b.x, b.y};
 }
+template <typename T>
+__device__ __forceinline__ T* slot_row(const Own1<T>& o, int plane, int t)
+{
+    return o.row() + 4 * (plane * (o.nt + 1) + t);
+}
+template <typename T> __device__ __forceinline__ T& slot_delta(const Own1<T>& o, int t) { return slot_row(o, 0, t)[3]; }
+template <typename T> __device__ __forceinline__ T& slot_gam(const Own1<T>& o, int t) { return slot_row(o, 1, t)[3]; }
+template <typename T> __device__ __forceinline__ T& slot_gref(const Own1<T>& o, int t) { return slot_row(o, 2, t)[3]; }
 
 template <typename T>
 __device__ __forceinline__ int slot_gid(const Own1<T>& o, int t)
@@ -1338,11 +1472,185 @@ __device__ __forceinline__ int slot_gid(const Own1<T>& o, int t)
     return t < o.nc ? o.c0 + t : o.gid[t - o.nc];
 }
 
-// Rod phase over the block's rods, every entry from shared memory (modes
-// as for phase_a: A_STEP forms delta_{k+1} with alpha and leaves dU in
-// shared memory; A_PG returns this thread's share of pi.A.pi; A_REF leaves
-// Uref = M D gamma_ref (compensated in float32) in shared memory and in
-// the global Uref).
+// Stage one slot (owned or ghost) of constraint c from the global arrays.
+template <typename T>
+__device__ __forceinline__ void stage_slot(const SolveArgs<T>& a, const Own1<T>& o, int t)
+{
+    const size_t mp = a.mp;
+    const int c = slot_gid(o, t);
+#pragma unroll
+    for (int w = 0; w < 9; ++w) slot_row(o, w / 3, t)[w % 3] = a.rec[w * mp + c];
+    T d, g, gr, gl;
+    ld_state(a.gg0, c, d, g, gr, gl);
+    slot_delta(o, t) = d;
+    slot_gam(o, t) = gr;
+    slot_gref(o, t) = gl;   // gamma_lo until the first reference pass replaces it
+}
+
+// Hash set of the halo's ranks while the share is staged, in the rows' space
+// (linear probing, at most half full: size is a power of two >= 2 nt).
+struct RankSet {
+    int* key;
+    int* val;
+    int size, shift;
+    __device__ __forceinline__ int first(int r) const { return (int)((unsigned)r * 2654435761u >> shift); }
+    __device__ __forceinline__ void insert(int r)
+    {
+        for (int h = first(r);; h = (h + 1) & (size - 1)) {
+            const int was = atomicCAS(&key[h], -1, r);
+            if (was == -1 || was == r) return;
+        }
+    }
+    __device__ __forceinline__ int find(int r) const
+    {
+        int h = first(r);
+        while (key[h] != r) h = (h + 1) & (size - 1);
+        return val[h];
+    }
+};
+
+template <typename T>
+__device__ __noinline__ void stage_in1(const SolveArgs<T>& a, Shared1<T>& sh)
+{
+    Own1<T>& o = sh.o;
+    const int nr = o.r1 - o.r0, nq = o.q1 - o.q0;
+    // ghosts: other-side entries of the block's rods that another block owns
+    if (threadIdx.x == 0) sh.ng = sh.ne = sh.nh = 0;
+    __syncthreads();
+    int cnt = 0, fours = 0;
+    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+        const int c = a.qlist[o.q0 + k];
+        cnt += c < o.c0 || c >= o.c1;
+    }
+    for (int i = o.r0 + threadIdx.x; i < o.r1; i += blockDim.x)
+        fours += (a.rowP[i + 1] - a.rowP[i] + a.rowQ[i + 1] - a.rowQ[i] + 3) >> 2;
+    if (cnt) atomicAdd(&sh.ng, cnt);
+    if (fours) atomicAdd(&sh.ne, 4 * fours);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        o.ng = sh.ng;
+        o.nt = o.nc + o.ng;
+        o.ne = sh.ne;
+        carve1(o);
+        o.gid = reinterpret_cast<int*>(a.gref) + o.q0;   // gref itself lives in the slots
+        o.hrank = a.hrank + o.c0 + o.q0;
+        sh.ng = 0;
+    }
+    __syncthreads();
+    RankSet set;
+    set.size = 2;
+    set.shift = 31;
+    while (set.size < 2 * o.nt) { set.size *= 2; --set.shift; }
+    set.key = reinterpret_cast<int*>(o.row());
+    set.val = set.key + set.size;   // 2 size <= 8 nt words (or 4) of the rows' 12 (nt + 1)
+    for (int h = threadIdx.x; h < set.size; h += blockDim.x) set.key[h] = -1;
+    // rod order by (owned, other-side) counts for the initial pass, whose
+    // per-thread sums depend on it; the keys and ranks live in the velocities'
+    // space, which the first pass fills
+    {
+        unsigned* key = reinterpret_cast<unsigned*>(o.U());
+        sort_rods(a.rowP + o.r0, a.rowQ + o.r0, nr, key, reinterpret_cast<int*>(key) + nr, o.perm());
+    }
+    if (threadIdx.x < 32) {   // first entry of every rod
+        int base = 0;
+        for (int l0 = 0; l0 <= nr; l0 += 32) {
+            const int li = l0 + (int)threadIdx.x, i = o.r0 + li;
+            const int f = li < nr ? (a.rowP[i + 1] - a.rowP[i] + a.rowQ[i + 1] - a.rowQ[i] + 3) >> 2 : 0;
+            int x = f;
+#pragma unroll
+            for (int s = 1; s < 32; s *= 2) {
+                const int y = __shfl_up_sync(0xffffffffu, x, s);
+                if ((int)threadIdx.x >= s) x += y;
+            }
+            if (li <= nr) o.rowE()[li] = (unsigned short)(base + x - f);
+            base += __shfl_sync(0xffffffffu, x, 31);
+        }
+    }
+    for (int li = threadIdx.x; li < nr; li += blockDim.x)
+        for (int w = 0; w < 3; ++w) o.ax()[w * o.cap_r + li] = a.ax[w * (size_t)a.np + o.r0 + li];
+    for (int e = threadIdx.x; e < o.ne; e += blockDim.x) o.ent()[e] = (unsigned short)o.nt;
+    // the halo: other ends of owned constraints, owners of ghosts
+    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) {
+        const int j = a.cj[o.c0 + t];
+        if (j >= 0 && (j < o.r0 || j >= o.r1)) set.insert(j);
+    }
+    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+        const int c = a.qlist[o.q0 + k];
+        if (c < o.c0 || c >= o.c1) set.insert(a.ci[c]);
+    }
+    __syncthreads();
+    for (int h = threadIdx.x; h < set.size; h += blockDim.x) {
+        if (set.key[h] >= 0) {
+            const int x = atomicAdd(&sh.nh, 1);   // (no result depends on the halo's order)
+            set.val[h] = x;
+            o.hrank[x] = set.key[h];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        o.nh = sh.nh;
+        carve_rest(o, a.dyn_bytes, a.priv, (size_t)a.mp);
+    }
+    const int zero = nr, halo = nr + 1;   // velocity rows: own rods, zero, halo
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) {
+        const int c = o.c0 + t, i = a.ci[c], j = a.cj[c], li = i - o.r0;
+        const int lj = j < 0 ? zero : j >= o.r0 && j < o.r1 ? j - o.r0 : halo + set.find(j);
+        o.ij()[t] = (unsigned)li | (unsigned)lj << 16;
+        o.ent()[4 * o.rowE()[li] + c - a.rowP[i]] = (unsigned short)t;
+    }
+    // other-side entries in CSR order
+#pragma unroll 1
+    for (int k = o.q0 + threadIdx.x; k < o.q1; k += blockDim.x) {
+        const int c = a.qlist[k], j = a.cj[c], li = j - o.r0;   // the block's rod is c's Q side
+        int t = c - o.c0;
+        if (c < o.c0 || c >= o.c1) {
+            // the slot order of ghosts does not enter any result
+            const int g = atomicAdd(&sh.ng, 1);
+            t = o.nc + g;
+            o.gid[g] = c;
+            o.ij()[t] = (unsigned)(halo + set.find(a.ci[c])) | (unsigned)li << 16;
+        }
+        o.ent()[4 * o.rowE()[li] + a.rowP[j + 1] - a.rowP[j] + k - a.rowQ[j]] = (unsigned short)(t | kOther);
+    }
+    __syncthreads();   // the rows take the place of the set
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) stage_slot(a, o, t);
+    if (threadIdx.x < 12) slot_row(o, threadIdx.x / 4, o.nt)[threadIdx.x % 4] = T(0);
+    if (threadIdx.x < 6) o.U()[6 * zero + threadIdx.x] = T(0);
+    __syncthreads();
+}
+
+// Orders the block's rods by the length of their entry loops, so that the
+// rods of a warp run about equally long: a counting sort (no result depends
+// on the order within one length) over kLens counters.
+constexpr int kLens = 64;
+template <typename T>
+__device__ __noinline__ void sort_rods_total(const Own1<T>& o, int* count)
+{
+    const int nr = o.r1 - o.r0, lane = threadIdx.x & 31;
+    if (threadIdx.x < kLens) count[threadIdx.x] = 0;
+    __syncthreads();
+    for (int li = threadIdx.x; li < nr; li += blockDim.x)
+        atomicAdd(&count[min(o.rowE()[li + 1] - o.rowE()[li], kLens - 1)], 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {   // starts of the lengths
+        const int c0 = count[2 * lane], c1 = count[2 * lane + 1];
+        int x = c0 + c1;
+#pragma unroll
+        for (int s = 1; s < 32; s *= 2) {
+            const int y = __shfl_up_sync(0xffffffffu, x, s);
+            if (lane >= s) x += y;
+        }
+        count[2 * lane] = x - c0 - c1;
+        count[2 * lane + 1] = x - c1;
+    }
+    __syncthreads();
+    for (int li = threadIdx.x; li < nr; li += blockDim.x)
+        o.perm()[atomicAdd(&count[min(o.rowE()[li + 1] - o.rowE()[li], kLens - 1)], 1)] = (unsigned short)li;
+    __syncthreads();
+}
+
 // The six low parts of one side of constraint c: e's, then the arm's (rec_lo
 // rows 0-2 and 3-5 for the owner, 0-2 and 6-8 for the other side, arm0 = 3
 // or 6), from the side's 32-byte row when there is one.
@@ -1363,108 +1671,198 @@ __device__ __forceinline__ void lo_side(const T* rows, const T* rec_lo, size_t m
     }
 }
 
+// Velocity M F of one rod, three components: a n F + p (p.F)(b - a), the
+// translational half (a = 1/zeta_perp, b = 1/zeta_par) or the rotational
+// one.  The products' fusing is written out, so that every kernel rounds alike.
+template <typename T>
+__device__ __forceinline__ void half_mobility(const T p[3], const T F[3], T ia, T ib, T U[3])
+{
+    const T pf = fma(p[2], F[2], fma(p[0], F[0], p[1] * F[1]));
+    const T cf = pf * (ib - ia);
+#pragma unroll
+    for (int w = 0; w < 3; ++w) U[w] = fma(p[w], cf, F[w] * ia);
+}
+
+// Rod pass of the reference (one thread per rod): A_REF leaves Uref = M D
+// gamma_ref (compensated in float32) in shared memory and in the global
+// Uref; A_PG returns this thread's share of pi.A.pi.
 template <typename T, int MODE>
-__device__ __forceinline__ T rod_pass1(const SolveArgs<T>& a, const Own1<T>& o, T alpha)
+__device__ __noinline__ T rod_pass1(const SolveArgs<T>& a, const Own1<T>& o)
 {
     constexpr bool COMP = MODE == A_REF && sizeof(T) == 4;
     const bool has_comp = a.comp != nullptr;
-    const size_t mp = a.mp, np = a.np, nt = o.nt;
+    const size_t mp = a.mp, np = a.np;
     T fmf = T(0);
 #pragma unroll 1
-    for (int tt = threadIdx.x; tt < o.r1 - o.r0; tt += blockDim.x) {
-        const int li = (int)o.perm[tt], i = o.r0 + li;
+    for (int tt = first_item(a); tt < o.r1 - o.r0; tt += a.workers) {
+        const int li = (int)o.perm()[tt], i = o.r0 + li;
         Acc<T, COMP> Fa[6];
 #pragma unroll
         for (int w = 0; w < 6; ++w) Fa[w].init(T(0));
-        {   // owned constraints: slots [rowP[li] - c0, rowP[li + 1] - c0)
-            const int e = o.rowP[li + 1] - o.c0;
+        const int e1 = 4 * o.rowE()[li + 1];
 #pragma unroll 1
-            for (int t = o.rowP[li] - o.c0; t < e; ++t) {
-                const T dv = o.ds[t], gv = o.grs[t], gr = o.gam[t];
-                T rv[6];
+        for (int e = 4 * o.rowE()[li]; e < e1; ++e) {   // owned constraints, then those other rods own
+            const unsigned x = o.ent()[e];
+            const int t = (int)(x & ~kOther);
+            if (t == o.nt) break;   // padding
+            const bool own = !(x & kOther);
+            const Row<T> re = ld_row(slot_row(o, 0, t)), rp = ld_row(slot_row(o, 1, t)), rq = ld_row(slot_row(o, 2, t));
+            const T r[6] = {re.x, re.y, re.z, own ? rp.x : rq.x, own ? rp.y : rq.y, own ? rp.z : rq.z};
+            const T g = rq.w;   // gref; gamma_lo during a refresh
+            const int c = slot_gid(o, t);
+            const T cmp = has_comp ? __ldg(&a.comp[c]) : T(-1);
+            const bool bil = cmp >= T(0);
+            const T v = a_value<MODE, T>(re.w, g, rp.w, T(0), bil);
+            if (MODE == A_PG && own && bil) fmf += cmp * v * v;   // the spring's compliance term
+            const T sv = own ? v : -v;
 #pragma unroll
-                for (int w = 0; w < 6; ++w) rv[w] = o.rec[w * nt + t];
-                const bool bil = has_comp && (o.loc[t] & kBil);
-                const T v = a_value<MODE, T>(dv, gv, gr, alpha, bil);
-                if (MODE == A_PG && bil) fmf += __ldg(&a.comp[o.c0 + t]) * v * v;   // the spring's compliance term
+            for (int w = 0; w < 6; ++w) Fa[w].add_prod(sv, r[w]);
+            if (COMP) {   // gamma_lo and the records' low parts
+                T rl[6];
+                lo_side(own ? a.lop : a.loq, a.rec_lo, mp, c, own ? 3 : 6, rl);
 #pragma unroll
-                for (int w = 0; w < 6; ++w) Fa[w].add_prod(v, rv[w]);
-                if (COMP) {   // gamma_lo (held in grs during a reference pass) and the records' low parts
-                    const int c = o.c0 + t;
-                    const T gl = gv;
-                    T rl[6];
-                    lo_side(a.lop, a.rec_lo, mp, c, 3, rl);
-#pragma unroll
-                    for (int w = 0; w < 6; ++w) Fa[w].add_lo(v * rl[w] + gl * rv[w]);
-                }
-            }
-        }
-        {   // constraints owned by other rods (owned or ghost slots)
-            const int e = o.rowQ[li + 1] - o.q0;
-#pragma unroll 1
-            for (int k = o.rowQ[li] - o.q0; k < e; ++k) {
-                const unsigned qs = o.qslot[k];
-                const int t = (int)(qs & kMaxSlots);
-                const T dv = o.ds[t], gv = o.grs[t], gr = o.gam[t];
-                T qv[6];
-#pragma unroll
-                for (int w = 0; w < 3; ++w) {
-                    qv[w] = o.rec[w * nt + t];
-                    qv[3 + w] = o.rec[(6 + w) * nt + t];
-                }
-                const T v = a_value<MODE, T>(dv, gv, gr, alpha, has_comp && (qs & kBil));
-#pragma unroll
-                for (int w = 0; w < 6; ++w) Fa[w].add_prod(-v, qv[w]);
-                if (COMP) {
-                    const int c = slot_gid(o, t);
-                    const T gl = gv;
-                    T ql[6];
-                    lo_side(a.loq, a.rec_lo, mp, c, 6, ql);
-#pragma unroll
-                    for (int w = 0; w < 6; ++w) Fa[w].add_lo(-(v * ql[w] + gl * qv[w]));
+                for (int w = 0; w < 6; ++w) {
+                    const T lo = fma(v, rl[w], g * r[w]);
+                    Fa[w].add_lo(own ? lo : -lo);
                 }
             }
         }
         T F[6];
 #pragma unroll
         for (int w = 0; w < 6; ++w) F[w] = Fa[w].value();
-        const T p0 = o.ax[li], p1 = o.ax[o.cap_r + li], p2 = o.ax[2 * o.cap_r + li];
+        const T p[3] = {o.ax()[li], o.ax()[o.cap_r + li], o.ax()[2 * o.cap_r + li]};
         T ip = a.inv_perp, ipa = a.inv_par, ir = a.inv_rot, is = a.inv_spin;
         if (a.mobr) {
             ip = __ldg(&a.mobr[i]); ipa = __ldg(&a.mobr[np + i]);
             ir = __ldg(&a.mobr[2 * np + i]); is = __ldg(&a.mobr[3 * np + i]);
         }
-        const T pf = p0 * F[0] + p1 * F[1] + p2 * F[2];
-        const T pt = p0 * F[3] + p1 * F[4] + p2 * F[5];
-        const T cf = pf * (ipa - ip), ct = pt * (is - ir);
-        const T Uv[6] = {F[0] * ip + p0 * cf, F[1] * ip + p1 * cf, F[2] * ip + p2 * cf,
-                         F[3] * ir + p0 * ct, F[4] * ir + p1 * ct, F[5] * ir + p2 * ct};
+        T Uv[6];
+        half_mobility(p, F, ip, ipa, Uv);
+        half_mobility(p, F + 3, ir, is, Uv + 3);
         if (MODE == A_PG) {
 #pragma unroll
             for (int w = 0; w < 6; ++w) fmf += F[w] * Uv[w];
         } else {
 #pragma unroll
-            for (int w = 0; w < 6; ++w) o.U[w * o.cap_r + li] = Uv[w];
-            if (MODE == A_REF) st_u6(a.Uref, i, Uv);
+            for (int w = 0; w < 6; ++w) o.U()[6 * li + w] = Uv[w];
+            st_u6(a.Uref, i, Uv);
         }
     }
     return fmf;
 }
 
-// The block's dU (shared [6][cap_r]) into its contiguous range of the
-// global [n][6] buffer dst, consecutive threads writing consecutive pairs.
-template <typename T>
-__device__ __forceinline__ void copy_out1(T* dst, const Own1<T>& o)
+// The sign of v flipped for an other-side entry.
+__device__ __forceinline__ float signed_by(float v, unsigned x)
 {
-    __syncthreads();
-    const int nr = o.r1 - o.r0;
-    typename V2<T>::t* g = reinterpret_cast<typename V2<T>::t*>(dst + 6 * (size_t)o.r0);
-    for (int k = threadIdx.x; k < 3 * nr; k += blockDim.x) {
-        const int r = k / 3, w = 2 * (k - 3 * r);
-        typename V2<T>::t v;
-        v.x = o.U[w * o.cap_r + r];
-        v.y = o.U[(w + 1) * o.cap_r + r];
-        g[k] = v;
+    return __uint_as_float(__float_as_uint(v) ^ (x & kOther) << 16);
+}
+__device__ __forceinline__ double signed_by(double v, unsigned x)
+{
+    return __hiloint2double(__double2hiint(v) ^ (int)((x & kOther) << 16), __double2loint(v));
+}
+
+// Rod phase of a step: dU = M D delta_{k+1}, two lanes per rod (force and
+// torque halves, which only meet in the slots), every entry from shared
+// memory: the slot's number, its delta, and one row.  The loads of four
+// entries are in flight together (the sums stay in entry order); dU goes to
+// shared memory and, tagged, to the other blocks.
+template <typename T>
+__device__ __forceinline__ void rod_step2(const SolveArgs<T>& a, const Own1<T>& o, uint4* xb, unsigned tag)
+{
+    const int n2 = 2 * (o.r1 - o.r0), r0 = o.r0, R = o.cap_r, plane = 4 * (o.nt + 1);
+    const T* const row = o.row();
+    const T* const ax = o.ax();
+    T* const Us = o.U();
+    const unsigned short *const perm = o.perm(), *const rowE = o.rowE();
+    const ushort4* const ent = reinterpret_cast<const ushort4*>(o.ent());
+#pragma unroll 1
+    for (int tt = first_item(a); tt < n2; tt += a.workers) {
+        const int li = (int)perm[tt >> 1], half = tt & 1;
+        const int e1 = rowE[li + 1];
+        const int own_plane = half ? plane : 0, oth_plane = half ? 2 * plane : 0;
+        T F[3] = {T(0), T(0), T(0)};
+#pragma unroll 1
+        for (int e = rowE[li]; e < e1; ++e) {
+            const ushort4 q = ent[e];
+            const unsigned x[4] = {q.x, q.y, q.z, q.w};
+            T v[4];
+            Row<T> r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const T* p = row + 4 * (int)(x[u] & ~kOther);
+                v[u] = signed_by(p[3], x[u]);
+                r[u] = ld_row(p + (x[u] & kOther ? oth_plane : own_plane));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                F[0] = fma(v[u], r[u].x, F[0]);
+                F[1] = fma(v[u], r[u].y, F[1]);
+                F[2] = fma(v[u], r[u].z, F[2]);
+            }
+        }
+        const int i = r0 + li;
+        const T p[3] = {ax[li], ax[R + li], ax[2 * R + li]};
+        T ia = half ? a.inv_rot : a.inv_perp, ib = half ? a.inv_spin : a.inv_par;
+        if (a.mobr) {
+            ia = __ldg(&a.mobr[(half ? 2 * (size_t)a.np : 0) + i]);
+            ib = __ldg(&a.mobr[(half ? 3 * (size_t)a.np : (size_t)a.np) + i]);
+        }
+        T U[3];
+        half_mobility(p, F, ia, ib, U);
+        Tagged<T, 3>::put(xb + Xch<T>::kWords * (size_t)i + half * Tagged<T, 3>::kWords, U, tag);
+#pragma unroll
+        for (int w = 0; w < 3; ++w) Us[6 * li + 3 * half + w] = U[w];
+    }
+}
+
+// The same with eight lanes per rod, one component each (two idle), for
+// shares of few rods, whose entry loops would otherwise leave most of the
+// block waiting for a warp or two.
+template <typename T>
+__device__ __forceinline__ void rod_step8(const SolveArgs<T>& a, const Own1<T>& o, uint4* xb, unsigned tag)
+{
+    const int nr = o.r1 - o.r0, r0 = o.r0, R = o.cap_r, plane = 4 * (o.nt + 1);
+    const T* const row = o.row();
+    const ushort4* const ent = reinterpret_cast<const ushort4*>(o.ent());
+    const int lane = threadIdx.x & 31, sub = lane & 7, half = sub >= 3, w = half ? (sub < 6 ? sub - 3 : 0) : sub;
+    const int own_off = (half ? plane : 0) + w, oth_off = (half ? 2 * plane : 0) + w;
+#pragma unroll 1
+    for (int tt = first_item(a) >> 3; (tt & ~3) < nr; tt += a.workers >> 3) {   // (uniform per warp)
+        const int li = (int)o.perm()[min(tt, nr - 1)];
+        const int e1 = tt < nr ? (int)o.rowE()[li + 1] : 0;
+        T F = T(0);
+#pragma unroll 1
+        for (int e = o.rowE()[li]; e < e1; ++e) {
+            const ushort4 q = ent[e];
+            const unsigned x[4] = {q.x, q.y, q.z, q.w};
+            T v[4], r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const T* p = row + 4 * (int)(x[u] & ~kOther);
+                v[u] = signed_by(p[3], x[u]);
+                r[u] = p[x[u] & kOther ? oth_off : own_off];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) F = fma(v[u], r[u], F);
+        }
+        __syncwarp();
+        const int i = r0 + li, g0 = (lane & 24) + (half ? 3 : 0);
+        const T* const ax = o.ax();
+        const T p[3] = {ax[li], ax[R + li], ax[2 * R + li]};
+        T Fh[3], U[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Fh[c] = __shfl_sync(0xffffffffu, F, g0 + c);
+        T ia = half ? a.inv_rot : a.inv_perp, ib = half ? a.inv_spin : a.inv_par;
+        if (a.mobr) {
+            ia = __ldg(&a.mobr[(half ? 2 * (size_t)a.np : 0) + i]);
+            ib = __ldg(&a.mobr[(half ? 3 * (size_t)a.np : (size_t)a.np) + i]);
+        }
+        half_mobility(p, Fh, ia, ib, U);
+        if (tt < nr && (sub == 0 || sub == 3)) {
+            Tagged<T, 3>::put(xb + Xch<T>::kWords * (size_t)i + half * Tagged<T, 3>::kWords, U, tag);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) o.U()[6 * li + 3 * half + c] = U[c];
+        }
     }
 }
 
@@ -1474,7 +1872,7 @@ template <typename T>
 __device__ __forceinline__ void zero_uref1(const SolveArgs<T>& a, const Own1<T>& o)
 {
     const int nr = o.r1 - o.r0;
-    for (int k = threadIdx.x; k < 6 * o.cap_r; k += blockDim.x) o.U[k] = T(0);
+    for (int k = threadIdx.x; k < 6 * o.cap_r; k += blockDim.x) o.U()[k] = T(0);
     typename V2<T>::t z;
     z.x = T(0);
     z.y = T(0);
@@ -1482,56 +1880,69 @@ __device__ __forceinline__ void zero_uref1(const SolveArgs<T>& a, const Own1<T>&
     for (int k = threadIdx.x; k < 3 * nr; k += blockDim.x) g[k] = z;
 }
 
-// The two velocities of slot t, P side first: Ui of the owner, Uj of the
-// other end (0 for a wall).  Local rods from shared memory, others from the
-// global buffer Ug.
+// A halo rod's velocity of exchange tag, polled.
 template <typename T>
-__device__ __forceinline__ void slot_velocities(const Own1<T>& o, int t, const T* Ug, T Ui[6], T Uj[6])
+__device__ __forceinline__ void get_halo(const SolveArgs<T>& a, const Own1<T>& o, int h, const uint4* xb, unsigned tag,
+                                         int* bad, T U[6])
 {
-    const int li = (int)(o.loc[t] & kMaxSlots);
-    const int ro = o.oth[t];
-    T Ul[6], Uo[6];
-#pragma unroll
-    for (int w = 0; w < 6; ++w) Ul[w] = o.U[w * o.cap_r + li];
-    if (ro < 0) {
-#pragma unroll
-        for (int w = 0; w < 6; ++w) Uo[w] = T(0);
-    } else if (ro >= o.r0 && ro < o.r1) {
-#pragma unroll
-        for (int w = 0; w < 6; ++w) Uo[w] = o.U[w * o.cap_r + (ro - o.r0)];
-    } else {
-        ld_u6(Ug, ro, Uo);
-    }
-    const bool own = t < o.nc;
-#pragma unroll
-    for (int w = 0; w < 6; ++w) {
-        Ui[w] = own ? Ul[w] : Uo[w];
-        Uj[w] = own ? Uo[w] : Ul[w];
+    get_tagged<T, 6>(a.flags, a.wait_cycles, xb + Xch<T>::kWords * (size_t)o.hrank[h], tag, bad, U);
+}
+
+// The halo's velocities of exchange tag into their rows, by the threads with
+// the fewest rods first, one rod polled at a time (polling two held the
+// publishers up: 2e4 rods 1.46 -> 1.71 ms).
+template <typename T>
+__device__ __forceinline__ void fetch_halo(const SolveArgs<T>& a, const Own1<T>& o, const uint4* xb, unsigned tag, int* bad)
+{
+    if (!o.halo || (int)threadIdx.x >= a.workers) return;
+    T* const Uh = o.U() + 6 * (o.cap_r + 1);
+#pragma unroll 1
+    for (int h = a.workers - 1 - (int)threadIdx.x; h < o.nh; h += a.workers) {
+        T U[6];
+        get_halo(a, o, h, xb, tag, bad, U);
+        st_u6(Uh, h, U);
     }
 }
 
-// Constraint phase of a step over every slot: delta_k from
-// (delta_{k-1}, g_{k-1}, alpha_{k-1}) exactly as the rod phase formed it,
-// g_k = gref + D^T dU_k (+ the spring's compliance term), and for owned
-// slots acc = (s.s, s.y, y.y, max |pi|).
-template <typename T>
-__device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1<T>& o, T alpha, const T* Ug, T acc[4])
+// Constraint phase of step k over every slot: from delta_k (which the rod
+// phase used), g_k = gref + D^T dU_k (+ the spring's compliance term), for
+// owned slots acc = (s.s, s.y, y.y, max |pi|), and delta_{k+1} =
+// max(-gamma_ref, delta_k - alpha_k g_k) for the rod phase.  POLL: the halo
+// has no rows, its velocities are polled here.
+template <typename T, bool POLL>
+__device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1<T>& o, T alpha, const uint4* xb,
+                                               unsigned tag, int* bad, T acc[4])
 {
     const bool has_comp = a.comp != nullptr;
-    const size_t nt = o.nt;
+    const int nt = o.nt, nc = o.nc, plane = 4 * (nt + 1), halo = o.cap_r + 1;
+    T* const row = o.row();
+    const T* const Us = o.U();
+    const unsigned* const ij = o.ij();
+    T *const ds = o.ds, *const gs = o.gs;
+    const T* const isc = a.isc + o.c0;
 #pragma unroll 1
-    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
-        T Ui[6], Uj[6], r[9];
-        slot_velocities(o, t, Ug, Ui, Uj);
-#pragma unroll
-        for (int w = 0; w < 9; ++w) r[w] = o.rec[w * nt + t];
-        const T dold = o.ds[t], gro = o.grs[t], gam = o.gam[t];
-        const int c = slot_gid(o, t);
-        const T cmp = has_comp ? __ldg(&a.comp[c]) : T(-1);
-        const bool bil = cmp >= T(0);
-        const T dm = a_value<A_STEP, T>(dold, gro, gam, alpha, bil);
+    for (int t = first_item(a); t < nt; t += a.workers) {
+        const unsigned x = ij[t];
+        const int i = (int)(x & 0xffffu), j = (int)(x >> 16);
+        T Ui[6], Uj[6];
+        T dold = T(0), gold = T(0), is = T(0);
+        if (t < nc) { dold = ds[t]; gold = gs[t]; is = __ldg(&isc[t]); }
+        if (POLL && i >= halo) get_halo(a, o, i - halo, xb, tag, bad, Ui);
+        else ld_u6(Us, i, Ui);
+        if (POLL && j >= halo) get_halo(a, o, j - halo, xb, tag, bad, Uj);
+        else ld_u6(Us, j, Uj);
+        T* const p = row + 4 * t;
+        const Row<T> re = ld_row(p), rp = ld_row(p + plane), rq = ld_row(p + 2 * plane);
+        const T dm = re.w, gam = rp.w;
+        T cmp = T(0);
+        bool bil = false;
+        if (has_comp) {
+            cmp = __ldg(&a.comp[slot_gid(o, t)]);
+            bil = cmp >= T(0);
+        }
         Acc<T, false> du;
-        du.init(o.gref[t]);
+        du.init(rq.w);
+        const T r[9] = {re.x, re.y, re.z, rp.x, rp.y, rp.z, rq.x, rq.y, rq.z};
 #pragma unroll
         for (int u = 0; u < 3; ++u) {
             du.add_prod(r[u], Ui[u]);
@@ -1541,13 +1952,14 @@ __device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1
         }
         if (bil) du.add_prod(cmp, dm);
         const T gr = du.value();
-        o.ds[t] = dm;
-        o.grs[t] = gr;
-        if (t < o.nc) {
+        p[3] = a_value<A_STEP, T>(dm, gr, gam, alpha, bil);
+        if (t < nc) {
+            ds[t] = dm;
+            gs[t] = gr;
             const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
-            const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
+            const T api = (pi < T(0) ? -pi : pi) * is;
             acc[3] = api > acc[3] ? api : acc[3];
-            const T sv = dm - dold, yv = gr - gro;
+            const T sv = dm - dold, yv = gr - gold;
             acc[0] += sv * sv;
             acc[1] += sv * yv;
             acc[2] += yv * yv;
@@ -1557,25 +1969,34 @@ __device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1
 
 // Constraint phase of a refresh over every slot: gref = q + D^T Uref from
 // the split records and q with compensated sums (float32), g = gref, and
-// for owned slots acc = (pi.pi, 0, 0, max |pi|) at gamma_ref.  ZERO: Uref
-// is 0 (gamma_ref = 0), so no velocity is read and the records' products
-// (all zero) are left out of the sums.
-template <typename T, bool ZERO = false>
-__device__ __forceinline__ void con_pass_ref1(const SolveArgs<T>& a, const Own1<T>& o, T acc[4])
+// for owned slots acc = (pi.pi, 0, 0, max |pi|) at gamma_ref; then, but in
+// the initial pass (whose step length is still to come), delta for the step
+// from the reference.  ZERO: the initial pass at gamma_0 = 0, where Uref is
+// 0, so no velocity is read and the records' products (all zero) are left
+// out of the sums.
+template <typename T, bool ZERO, bool INITIAL>
+__device__ __noinline__ void con_pass_ref1(const SolveArgs<T>& a, const Own1<T>& o, T alpha, T& sum_out, T& max_out)
 {
+    T acc[4] = {T(0), T(0), T(0), T(0)};
     constexpr bool COMP = sizeof(T) == 4;
     const bool has_comp = a.comp != nullptr;
-    const size_t nt = o.nt, mp = a.mp;
+    const size_t mp = a.mp;
+    const int halo = o.cap_r + 1;
 #pragma unroll 1
-    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
+    for (int t = first_item(a); t < o.nt; t += a.workers) {
         T Ui[6], Uj[6], r[9];
         if (!ZERO) {
-            slot_velocities(o, t, a.Uref, Ui, Uj);
+            const unsigned x = o.ij()[t];
+            const int i = (int)(x & 0xffffu), j = (int)(x >> 16);
+            if (i >= halo) ld_u6(a.Uref, o.hrank[i - halo], Ui);
+            else ld_u6(o.U(), i, Ui);
+            if (j >= halo) ld_u6(a.Uref, o.hrank[j - halo], Uj);
+            else ld_u6(o.U(), j, Uj);
 #pragma unroll
-            for (int w = 0; w < 9; ++w) r[w] = o.rec[w * nt + t];
+            for (int w = 0; w < 9; ++w) r[w] = slot_row(o, w / 3, t)[w % 3];
         }
         const int c = slot_gid(o, t);
-        const T gam = o.gam[t];
+        const T gam = slot_gam(o, t);
         Acc<T, COMP> du;
         du.init(__ldg(&a.q[c]));
         if (!ZERO) {
@@ -1591,7 +2012,7 @@ __device__ __forceinline__ void con_pass_ref1(const SolveArgs<T>& a, const Own1<
         const bool bil = cmp >= T(0);
         if (bil) {
             du.add_prod(cmp, gam);
-            du.add_lo(cmp * o.grs[t]);   // gamma_lo, before g takes its place below
+            du.add_lo(cmp * slot_gref(o, t));   // gamma_lo, before gref takes its place below
         }
         if (COMP) {
             T tl = __ldg(&a.q_lo[c]);
@@ -1601,39 +2022,52 @@ __device__ __forceinline__ void con_pass_ref1(const SolveArgs<T>& a, const Own1<
                 lo_side(a.loq, a.rec_lo, mp, c, 6, lq);
 #pragma unroll
                 for (int u = 0; u < 3; ++u)
-                    tl += lp[u] * (Ui[u] - Uj[u]) + lp[3 + u] * Ui[3 + u] - lq[3 + u] * Uj[3 + u];
+                    tl += fma(-lq[3 + u], Uj[3 + u], fma(lp[u], Ui[u] - Uj[u], lp[3 + u] * Ui[3 + u]));
             }
             du.add_lo(tl);
         }
         const T gr = du.value();
-        o.gref[t] = gr;
-        o.grs[t] = gr;
+        const T dm = slot_delta(o, t);   // 0 after the fold
+        slot_gref(o, t) = gr;
+        if (!INITIAL) slot_delta(o, t) = a_value<A_STEP, T>(dm, gr, gam, alpha, bil);
         if (t < o.nc) {
-            const T dm = o.ds[t];   // 0 after the fold
             const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
             const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
             acc[3] = api > acc[3] ? api : acc[3];
             acc[0] += pi * pi;
+            o.ds[t] = dm;
+            o.gs[t] = gr;
         }
+    }
+    sum_out = acc[0];
+    max_out = acc[3];
+}
+
+// delta_1 of every slot, once alpha_0 is known.
+template <typename T>
+__device__ __noinline__ void first_step1(const SolveArgs<T>& a, const Own1<T>& o, T alpha)
+{
+    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
+        const bool bil = a.comp && __ldg(&a.comp[slot_gid(o, t)]) >= T(0);
+        slot_delta(o, t) = a_value<A_STEP, T>(slot_delta(o, t), slot_gref(o, t), slot_gam(o, t), alpha, bil);
     }
 }
 
 // Refresh, first half: every slot folds delta into (gamma_ref, gamma_lo)
 // as fold_delta does, from the previous reference's gamma_lo in gprev;
 // ghosts repeat their owner's arithmetic on the same inputs, so both hold
-// the same reference without waiting for each other.  gamma_ref goes to
-// gam, gamma_lo to grs (the reference passes' low part, until the constraint
-// pass replaces it by g), and owned slots publish (gamma_ref, gamma_lo) in
+// the same reference without waiting for each other.  gamma_lo goes to the
+// place of gref (the reference passes' low part, until the constraint
+// pass replaces it), and owned slots publish (gamma_ref, gamma_lo) in
 // gnew, the other state buffer (ghosts are still reading gprev).
 template <typename T>
-__device__ __forceinline__ void fold1(const SolveArgs<T>& a, const Own1<T>& o, const T* gprev, T* gnew)
+__device__ __noinline__ void fold1(const SolveArgs<T>& a, const Own1<T>& o, const T* gprev, T* gnew)
 {
-    const bool has_comp = a.comp != nullptr;
 #pragma unroll 1
     for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
         const int c = slot_gid(o, t);
-        const T d = o.ds[t], gr = o.gam[t], gl = gl_of_state(gprev, c);
-        const bool bil = has_comp && (o.loc[t] & kBil);
+        const T d = slot_delta(o, t), gr = slot_gam(o, t), gl = gl_of_state(gprev, c);
+        const bool bil = a.comp && __ldg(&a.comp[c]) >= T(0);
         T hi = T(0), lo = T(0);
         if (bil || d > -gr) {
             T s, e;
@@ -1643,58 +2077,51 @@ __device__ __forceinline__ void fold1(const SolveArgs<T>& a, const Own1<T>& o, c
             lo = l - (hi - s);
             if (!bil && (hi < T(0) || (hi == T(0) && lo < T(0)))) { hi = T(0); lo = T(0); }
         }
-        o.gam[t] = hi;
-        o.grs[t] = lo;
-        o.ds[t] = T(0);
+        slot_gam(o, t) = hi;
+        slot_gref(o, t) = lo;
+        slot_delta(o, t) = T(0);
         if (t < o.nc) st_ref(gnew, c, hi, lo);
     }
 }
 
-// cp.async of the last barrier's block sums ([4][nbp] of buffer src) into
-// shared memory; the threads that issue it wait for it in tot_wait.
+// Warp w's share of the block sums: each warp's (sum, sum, sum, max) into
+// red[w].  The four values fold into one register per lane as the tree
+// halves (lanes keep one value and pass the other on), so the five levels
+// cost six exchanges instead of twenty; every pair of operands is the same
+// as in a plain tree per value, and so is every bit.
 template <typename T>
-__device__ __forceinline__ void tot_fetch(const Own1<T>& o, const T* src)
+__device__ __forceinline__ void warp_partial(const T v[4], T (*red)[4])
 {
-    const int chunks = (int)(4 * (size_t)o.nbp * sizeof(T) / 16);
-    if ((int)threadIdx.x < chunks) {
-        for (int q = threadIdx.x; q < chunks; q += blockDim.x) {
-            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(o.tot) + 16 * (size_t)q);
-            const unsigned char* s = reinterpret_cast<const unsigned char*>(src) + 16 * (size_t)q;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(s) : "memory");
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-}
-__device__ __forceinline__ void tot_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// Warp w's share of the block sums: each warp's (sum, sum, sum, max) into red[w].
-template <typename T>
-__device__ __forceinline__ void warp_partial(T v[4], T (*red)[4])
-{
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    // value 0 (sum) stays in lanes 0-15, value 1 (sum) in lanes 16-31; likewise 2 (sum), 3 (max)
+    const T s01 = __shfl_xor_sync(all, h16 ? v[0] : v[1], 16);
+    const T s23 = __shfl_xor_sync(all, h16 ? v[2] : v[3], 16);
+    const T a = (h16 ? v[1] : v[0]) + s01;
+    const T b = h16 ? max_of(s23, v[3]) : v[2] + s23;
+    // the maximum ends in lanes 24-31, the sums in lanes 0, 16 and 8
+    const bool is_max = h16 && h8;
+    T x = h8 ? b : a;
+    T y = __shfl_xor_sync(all, h8 ? a : b, 8);
+    x = is_max ? max_of(y, x) : x + y;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int u = 0; u < 3; ++u) v[u] += __shfl_down_sync(0xffffffffu, v[u], o);
-        const T mx = __shfl_down_sync(0xffffffffu, v[3], o);
-        v[3] = mx > v[3] ? mx : v[3];
+    for (int o = 4; o > 0; o >>= 1) {
+        y = __shfl_xor_sync(all, x, o);
+        const bool up = lane & o;
+        x = is_max ? max_of(up ? y : x, up ? x : y) : x + y;
     }
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) red[threadIdx.x >> 5][u] = v[u];
-    }
+    if ((lane & 7) == 0) red[threadIdx.x >> 5][h8 ? (h16 ? 3 : 2) : (h16 ? 1 : 0)] = x;
 }
 
-// Warp 0 after a block barrier: the block's sums over red, lane 0 stores
-// them in dst ([4][stride]).
+// One warp after a block barrier: the block's sums over the workers' red;
+// lane 0 holds them.
 template <typename T>
-__device__ __forceinline__ void block_store(T (*red)[4], T* dst, int stride)
+__device__ __forceinline__ void block_sums1(T (*red)[4], int nw, T w[4])
 {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    T w[4] = {T(0), T(0), T(0), T(0)};
-    if (lane < nw) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = red[lane][u];
-    }
+    for (int u = 0; u < 4; ++u) w[u] = lane < nw ? red[lane][u] : T(0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
@@ -1702,53 +2129,93 @@ __device__ __forceinline__ void block_store(T (*red)[4], T* dst, int stride)
         const T mx = __shfl_down_sync(0xffffffffu, w[3], o);
         w[3] = mx > w[3] ? mx : w[3];
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) dst[u * stride + blockIdx.x] = w[u];
-    }
 }
 
-// One warp: the grid total of row u of the fetched block sums (sums for
-// u < 3, the maximum for u = 3), in a fixed order, so every block gets the
-// same numbers; every lane returns it.
+// One warp: the grid totals of the tagged block sums at sums ([nb], the
+// exchange's slot) in a fixed order, so every block gets the same numbers;
+// every lane returns them.  The words of several blocks are in flight
+// together.
 template <typename T>
-__device__ __forceinline__ T row_total(const Own1<T>& o, int nb, int u)
+__device__ __forceinline__ void grid_sums1(const SolveArgs<T>& a, const uint4* sums, int nb, unsigned tag, int* bad,
+                                           T w[4])
 {
+    constexpr int B = sizeof(T) == 4 ? 5 : 2;
     const int lane = threadIdx.x & 31;
-    const T* row = o.tot + (size_t)u * o.nbp;
-    T w = T(0);
-    for (int b = lane; b < nb; b += 32) {
-        const T x = row[b];
-        w = u == 3 ? (x > w ? x : w) : w + x;
+    w[0] = w[1] = w[2] = w[3] = T(0);
+    for (int b0 = lane; b0 < nb; b0 += 32 * B) {
+        T x[B][4];
+        unsigned late = 0;
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (b0 + 32 * u < nb && !XchSum<T>::get(sums + kSumWords * (size_t)(b0 + 32 * u), tag, x[u])) late |= 1u << u;
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            if (b0 + 32 * u >= nb) break;
+            if (late & (1u << u))
+                get_tagged<T, 4>(a.flags, a.wait_cycles, sums + kSumWords * (size_t)(b0 + 32 * u), tag, bad, x[u]);
+            w[0] += x[u][0];
+            w[1] += x[u][1];
+            w[2] += x[u][2];
+            w[3] = x[u][3] > w[3] ? x[u][3] : w[3];
+        }
     }
+    __syncwarp();
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) {
-        const T y = __shfl_xor_sync(0xffffffffu, w, s);
-        w = u == 3 ? (y > w ? y : w) : w + y;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) w[u] += __shfl_xor_sync(0xffffffffu, w[u], s);
+        const T y = __shfl_xor_sync(0xffffffffu, w[3], s);
+        w[3] = y > w[3] ? y : w[3];
     }
-    return w;
 }
 
-// The four totals, one warp each: warps 1-4 store them in shared memory and
-// meet on a named barrier (warp 0 meanwhile stores the block's own sums).
-template <typename T>
-__device__ __forceinline__ void warps_totals(const Own1<T>& o, int nb, T* tot)
-{
-    const int u = (int)(threadIdx.x >> 5) - 1;
-    const T w = row_total(o, nb, u);
-    if ((threadIdx.x & 31) == 0) tot[u] = w;
-    asm volatile("bar.sync 1, 128;\n" ::: "memory");
-}
-
-// Loop states: what the last constraint phase was (its sums are what the
-// last barrier published), and the decision taken for the next rod phase.
+// What an iteration published (its sums decide the next one's step), and
+// the decision taken for an iteration.
 enum { C_NONE1 = 0, C_STEP1 = 1, C_REF1 = 2 };
 enum { K_STEP1 = 0, K_REF1 = 1, K_STOP1 = 2 };
 
+// The decision for the next iteration, by one lane of each block (every
+// block decides alike on the same totals); cpub: what the sums are of.
 template <typename T>
-__global__ void __launch_bounds__(1024, 1) k_bbpgd1(SolveArgs<T> a)
+__device__ __forceinline__ void decide1(const SolveArgs<T>& a, Shared1<T>& sh, int cpub, const T tot[4])
 {
-    extern __shared__ __align__(16) unsigned char dyn[];
+    int k = sh.k + 1, next = K_STEP1;
+    T an = sh.alpha;
+    if (cpub == C_STEP1) {
+        // sums of the step before the one just formed, and max |pi| at the iterate before the slots'
+        sh.pimax = tot[3];
+        const int since = ++sh.since;
+        const bool below = !above_tol(a, tot[3]);
+        if ((below && since >= 2) || (a.refresh > 0 && since >= a.refresh) || k >= a.max_iter) {
+            next = K_REF1;
+        } else {
+            const T ss = tot[0], sy = tot[1], yy = tot[2];
+            an = (sh.hist & 1) == 0 ? ss / sy : sy / yy;
+            if (!(sy > T(0)) || !isfinite(an) || !(an > T(0))) an = sh.alpha0;
+            ++sh.hist;
+        }
+    } else if (cpub == C_REF1) {
+        // the fresh reference's exact residual: the step formed from it is dropped on a stop
+        sh.pimax = tot[3];
+        sh.since = 0;
+        if (!above_tol(a, tot[3]) || k - 1 >= a.max_iter) {
+            next = K_STOP1;
+            --k;
+        }
+    } else if (k >= a.max_iter) {
+        next = K_REF1;   // the cap reached before any step's sums came back
+    }
+    sh.k = k;
+    sh.alpha = an;
+    sh.kind = next;
+}
+
+// MAXT: the most threads of a launch (kThreads1: the default shape and its
+// further warp, with 72 registers a thread; 1024: every other shape).
+constexpr int kThreads1 = 800;
+template <typename T, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ SolveArgs<T> a)
+{
     __shared__ Shared1<T> sh;
     if (a.need1_dev) {
         // recorded step: every block reads the same need, so either all run
@@ -1760,28 +2227,43 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd1(SolveArgs<T> a)
         }
     }
     if (a.fault == 1 && blockIdx.x == 0) return;   // test hook: this block never arrives
-    Own1<T> o;
-    o.r0 = a.bstart[blockIdx.x];
-    o.r1 = a.bstart[blockIdx.x + 1];
-    o.c0 = a.rowP[o.r0];
-    o.c1 = a.rowP[o.r1];
-    o.q0 = a.rowQ[o.r0];
-    o.q1 = a.rowQ[o.r1];
-    o.nc = o.c1 - o.c0;
-    o.cap_r = o.r1 - o.r0;
-    const int nb = (int)gridDim.x;
-    o.nbp = (nb + 3) & ~3;
-    stage_in1(a, o, dyn, sh);
-    T* part = reinterpret_cast<T*>(a.partials);   // [2][4][nbp]
-    const size_t pstride = 4 * (size_t)o.nbp;
-    unsigned epoch = 0;
-    int* s_ok = &sh.ng;   // the barrier's broadcast word (ng is not needed after staging)
-    auto barrier = [&]() { return grid_barrier(a.bar, (unsigned)nb * ++epoch, a.flags, a.wait_cycles, s_ok); };
-    const int warp = threadIdx.x >> 5;
-    // step state, kept by thread 32 (warp 1, lane 0)
-    T alpha0 = T(1), pimax = T(0);
-    int k = 0, since = 0, hist = 0;
-    bool ok = true;
+    Own1<T>& o = sh.o;
+    if (threadIdx.x == 0) {
+        o.r0 = a.bstart[blockIdx.x];
+        o.r1 = a.bstart[blockIdx.x + 1];
+        o.c0 = a.rowP[o.r0];
+        o.c1 = a.rowP[o.r1];
+        o.q0 = a.rowQ[o.r0];
+        o.q1 = a.rowQ[o.r1];
+        o.nc = o.c1 - o.c0;
+        o.cap_r = o.r1 - o.r0;
+        sh.bad = 0;
+        sh.alpha0 = T(1);
+        sh.pimax = T(0);
+        sh.k = sh.since = sh.hist = sh.nref = 0;
+        sh.epoch = 0;
+    }
+    __syncthreads();
+    // the blocks' tagged sums ([kSumSlots][blocks][kSumWords])
+    auto sums = [&](unsigned tag) {
+        return a.xch + 2 * Xch<T>::kWords * (size_t)a.n + (size_t)(tag % kSumSlots) * gridDim.x * kSumWords;
+    };
+    {   // tags of earlier solves away: nobody polls before the first grid barrier
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        const size_t w0 = Xch<T>::kWords * (size_t)o.r0, w1 = Xch<T>::kWords * (size_t)o.r1;
+        for (size_t w = w0 + threadIdx.x; w < w1; w += blockDim.x) {
+            a.xch[w] = z;
+            a.xch[Xch<T>::kWords * (size_t)a.n + w] = z;
+        }
+        for (int w = threadIdx.x; w < kSumSlots * kSumWords; w += blockDim.x)
+            sums(w / kSumWords)[blockIdx.x * kSumWords + w % kSumWords] = z;
+    }
+    stage_in1(a, sh);
+    auto barrier = [&]() {
+        if (threadIdx.x == 0) ++sh.epoch;
+        return grid_barrier(a.bar, gridDim.x * sh.epoch, a.flags, a.wait_cycles, &sh.ng);
+    };
+    const bool duty = (threadIdx.x >> 5) == (blockDim.x >> 5) - 1;   // sums and decisions
 
     // initial reference at gamma_0 and the line step alpha_0 = pi.pi / pi.A.pi;
     // from gamma_0 = 0, Uref = M D gamma_0 = 0 needs no rod pass and no
@@ -1790,124 +2272,113 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd1(SolveArgs<T> a)
         zero_uref1(a, o);
         __syncthreads();
     } else {
-        rod_pass1<T, A_REF>(a, o, T(0));
-        ok = barrier();
+        rod_pass1<T, A_REF>(a, o);
+        if (!barrier()) return;
     }
-    int pw = 0;   // block-sum buffer the next barrier publishes
-    if (ok) {
+    {
+        const int nb = (int)gridDim.x, nbp = (nb + 3) & ~3, lane = threadIdx.x & 31;
+        T* const part = reinterpret_cast<T*>(a.partials);   // [4][nbp]
         T v[4] = {T(0), T(0), T(0), T(0)};
-        if (a.zero_start) con_pass_ref1<T, true>(a, o, v);
-        else con_pass_ref1(a, o, v);
-        __syncthreads();   // gref and g of every slot before the line step reads them
-        v[1] = rod_pass1<T, A_PG>(a, o, T(0));
-        warp_partial(v, sh.red);
+        T s0, s3;
+        if (a.zero_start) con_pass_ref1<T, true, true>(a, o, T(0), s0, s3);
+        else con_pass_ref1<T, false, true>(a, o, T(0), s0, s3);
+        v[0] = s0;
+        v[3] = s3;
+        __syncthreads();   // gref of every slot before the line step reads it
+        v[1] = rod_pass1<T, A_PG>(a, o);
+        if ((int)threadIdx.x < a.workers) warp_partial(v, sh.red);
         __syncthreads();
-        if (warp == 0) block_store(sh.red, part + pw * pstride, o.nbp);
-        ok = barrier();
-    }
-    if (ok) {
-        tot_fetch(o, part + pw * pstride);
-        tot_wait();
-        __syncthreads();
-        if (warp >= 1 && warp <= 4) {
-            warps_totals(o, nb, sh.tot);
-            const T* tot = sh.tot;
-            if (threadIdx.x == 32) {
-                pimax = tot[3];
+        if (duty) {
+            T w[4];
+            block_sums1(sh.red, a.workers >> 5, w);
+            if (lane == 0) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) part[u * nbp + blockIdx.x] = w[u];
+            }
+        }
+        __syncthreads();   // red is read
+        sort_rods_total(o, reinterpret_cast<int*>(sh.red));
+        if (!barrier()) return;
+        if (duty) {
+            T tot[4] = {T(0), T(0), T(0), T(0)};
+            for (int b = lane; b < nb; b += 32) {
+#pragma unroll
+                for (int u = 0; u < 3; ++u) tot[u] += __ldcg(&part[u * nbp + b]);
+                tot[3] = max_of(tot[3], __ldcg(&part[3 * nbp + b]));
+            }
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) {
+#pragma unroll
+                for (int u = 0; u < 3; ++u) tot[u] += __shfl_xor_sync(0xffffffffu, tot[u], s);
+                tot[3] = max_of(tot[3], __shfl_xor_sync(0xffffffffu, tot[3], s));
+            }
+            if (lane == 0) {
+                sh.pimax = tot[3];
                 const double pap = (double)tot[1];
                 double al = (double)tot[0] / pap;
                 if (!(pap > 0.0) || !isfinite(al) || !(al > 0.0) || !isfinite((T)al)) al = 1.0;
-                alpha0 = (T)al;
-                sh.alpha = alpha0;
-                sh.kind = (!above_tol(a, pimax) || a.max_iter <= 0) ? K_STOP1 : K_STEP1;
+                sh.alpha0 = sh.alpha = (T)al;
+                sh.kind = (!above_tol(a, tot[3]) || a.max_iter <= 0) ? K_STOP1 : K_STEP1;
             }
         }
         __syncthreads();
-        pw ^= 1;
     }
-    int cprev = C_NONE1;      // the constraint phase whose sums the last barrier published
-    bool rstep = false;       // the last rod phase formed a step (its delta is still to be stored)
-    T alpha_prev = T(0);
-    int db = 0;               // dU buffer the next step's rod phase writes
-    int nref = 0;             // refreshes taken: the reference lives in state buffer nref & 1
-    while (ok && sh.kind != K_STOP1) {
-        const int pr = pw ^ 1;   // buffer the last barrier published
-        if (cprev != C_NONE1) tot_fetch(o, part + pr * pstride);
-        T v[4] = {T(0), T(0), T(0), T(0)};
-        if (rstep) con_pass_step1(a, o, alpha_prev, db ? a.U : a.U2, v);
-        const int ccur = rstep ? C_STEP1 : C_NONE1;
-        warp_partial(v, sh.red);
-        tot_wait();
+    if (sh.kind != K_STOP1) {
+        first_step1(a, o, sh.alpha);
         __syncthreads();
-        if (warp == 0) {
-            block_store(sh.red, part + pw * pstride, o.nbp);
-        } else if (warp <= 4) {
-            if (cprev != C_NONE1) warps_totals(o, nb, sh.tot);
-            const T* tot = sh.tot;
-            if (threadIdx.x == 32) {
-                if (rstep) ++k;
-                int kind = K_STEP1;
-                T an = sh.alpha;
-                if (cprev == C_STEP1) {
-                    // sums of (s_{k-2}, y_{k-2}) and max |pi| at the iterate before the slots'
-                    pimax = tot[3];
-                    ++since;
-                    const bool below = !above_tol(a, pimax);
-                    if ((below && since >= 2) || (a.refresh > 0 && since >= a.refresh) || k >= a.max_iter) {
-                        kind = K_REF1;
-                    } else {
-                        const T ss = tot[0], sy = tot[1], yy = tot[2];
-                        an = (hist & 1) == 0 ? ss / sy : sy / yy;
-                        if (!(sy > T(0)) || !isfinite(an) || !(an > T(0))) an = alpha0;
-                        ++hist;
-                    }
-                } else if (cprev == C_REF1) {
-                    // the fresh reference's exact residual: the slots' step from it is dropped on a stop
-                    pimax = tot[3];
-                    since = 0;
-                    if (!above_tol(a, pimax) || k - 1 >= a.max_iter) {
-                        kind = K_STOP1;
-                        --k;
-                    }
-                } else if (k >= a.max_iter) {
-                    kind = K_REF1;   // the cap reached before any step's sums came back
-                }
-                sh.alpha = an;
-                sh.kind = kind;
+    }
+    unsigned tag = 0;         // exchanges so far: dU and sums of the last iteration carry it
+    while (sh.kind != K_STOP1) {
+        const uint4* const xr = a.xch + (tag & 1u) * (Xch<T>::kWords * (size_t)a.n);
+        int cpub = C_NONE1;   // what this iteration publishes
+        if (tag > 0) {   // the first iteration is the step from gamma_0, already formed
+            T v[4] = {T(0), T(0), T(0), T(0)};
+            if (sh.kind == K_REF1) {
+                fold1(a, o, sh.nref & 1 ? a.gg1 : a.gg0, sh.nref & 1 ? a.gg0 : a.gg1);
+                __syncthreads();
+                if (threadIdx.x == 0) ++sh.nref;
+                rod_pass1<T, A_REF>(a, o);
+                if (!barrier()) return;
+                T s0, s3;   // (v itself stays in registers)
+                con_pass_ref1<T, false, false>(a, o, sh.alpha, s0, s3);
+                v[0] = s0;
+                v[3] = s3;
+                cpub = C_REF1;
+            } else {
+                if (o.halo) con_pass_step1<T, false>(a, o, sh.alpha, xr, tag, &sh.bad, v);
+                else con_pass_step1<T, true>(a, o, sh.alpha, xr, tag, &sh.bad, v);
+                cpub = C_STEP1;
             }
-        }
-        __syncthreads();
-        const int kind = sh.kind;
-        if (kind == K_STOP1) break;
-        int cpub = ccur;
-        if (kind == K_REF1) {
-            fold1(a, o, nref & 1 ? a.gg1 : a.gg0, nref & 1 ? a.gg0 : a.gg1);
-            ++nref;
+            if ((int)threadIdx.x < a.workers) {
+                // (the sums of a warp without owned slots are zero)
+                if ((int)(threadIdx.x & ~31u) < o.nc) warp_partial(v, sh.red);
+                else if ((threadIdx.x & 31) < 4) sh.red[threadIdx.x >> 5][threadIdx.x & 3] = T(0);
+            }
             __syncthreads();
-            rod_pass1<T, A_REF>(a, o, T(0));
-            if (!(ok = barrier())) break;
-            T w[4] = {T(0), T(0), T(0), T(0)};
-            con_pass_ref1(a, o, w);
-            warp_partial(w, sh.red);
-            __syncthreads();
-            if (warp == 0) block_store(sh.red, part + pw * pstride, o.nbp);
-            cpub = C_REF1;
+            if (sh.bad) return;
         }
-        const T al = sh.alpha;
-        rod_pass1<T, A_STEP>(a, o, al);
-        copy_out1(db ? a.U2 : a.U, o);
-        alpha_prev = al;
-        rstep = true;
-        db ^= 1;
-        if (!(ok = barrier())) break;
-        pw ^= 1;
-        cprev = cpub;
+        ++tag;
+        if (duty && cpub != C_NONE1) {   // this block's sums, while the others run the rod phase
+            T w[4];
+            block_sums1(sh.red, a.workers >> 5, w);
+            if ((threadIdx.x & 31) == 0) XchSum<T>::put(sums(tag) + kSumWords * blockIdx.x, w, tag);
+        }
+        uint4* const xw = a.xch + (tag & 1u) * (Xch<T>::kWords * (size_t)a.n);
+        if (8 * (o.r1 - o.r0) <= a.workers) rod_step8(a, o, xw, tag);
+        else rod_step2(a, o, xw, tag);
+        fetch_halo(a, o, xw, tag, &sh.bad);
+        if (duty) {   // the next iteration's step
+            T tot[4];
+            if (cpub != C_NONE1) grid_sums1(a, sums(tag), (int)gridDim.x, tag, &sh.bad, tot);
+            if ((threadIdx.x & 31) == 0) decide1(a, sh, cpub, tot);
+        }
+        __syncthreads();   // dU and the decision before the next constraint phase
+        if (sh.bad) return;
     }
-    if (!ok) return;
     // every solve ends on a fresh reference: gamma = gamma_ref + gamma_lo
     // (state buffer nref & 1) and delta = 0, so dU = 0
-    T* gfin = nref & 1 ? a.gg1 : a.gg0;
-    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) st_dg(gfin, o.c0 + t, T(0), o.gref[t]);
+    T* gfin = sh.nref & 1 ? a.gg1 : a.gg0;
+    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) st_dg(gfin, o.c0 + t, T(0), slot_gref(o, t));
     {
         typename V2<T>::t z;
         z.x = T(0);
@@ -1915,11 +2386,11 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd1(SolveArgs<T> a)
         typename V2<T>::t* g = reinterpret_cast<typename V2<T>::t*>(a.U + 6 * (size_t)o.r0);
         for (int q = threadIdx.x; q < 3 * (o.r1 - o.r0); q += blockDim.x) g[q] = z;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 32) {
-        a.out[1] = (double)alpha0;
-        a.flags[F_FINAL] = nref & 1;
-        a.flags[F_ITERS] = k;
-        a.out[0] = a.hD * (double)pimax;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.out[1] = (double)sh.alpha0;
+        a.flags[F_FINAL] = sh.nref & 1;
+        a.flags[F_ITERS] = sh.k;
+        a.out[0] = a.hD * (double)sh.pimax;
     }
 }
 
@@ -2158,11 +2629,16 @@ static SolveArgs<T> make_args(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, int
     a.n = n; a.m = m; a.np = (int)ctx->max_rods; a.mp = (int)ctx->max_pairs;
     a.rowP = ctx->rowP; a.rowQ = ctx->rowQ; a.qlist = ctx->qlist; a.ci = ctx->ci; a.cj = ctx->cj;
     a.rec = sb.rec; a.qe = sb.qe; a.q = sb.q; a.ax = sb.ax;
-    a.gg0 = sb.gg[0]; a.gg1 = sb.gg[1]; a.U = sb.U; a.U2 = sb.U2; a.Uref = sb.Uref; a.gref = sb.gref;
+    a.gg0 = sb.gg[0]; a.gg1 = sb.gg[1]; a.U = sb.U; a.Uref = sb.Uref; a.gref = sb.gref;
     // float32 iterations work on increments over a reference that takes
     // the iterate every kRefresh iterations (and to confirm convergence);
     // float64 needs no refresh
     a.refresh = sizeof(T) == 4 ? kRefresh : 0;
+    a.xch = ctx->xch;
+    a.priv = sb.priv;
+    a.hrank = sb.hrank;
+    a.dyn_bytes = 0;
+    a.workers = ctx->solve_threads;
     a.partials = ctx->partials; a.bar = ctx->bar; a.flags = ctx->dflags;
     a.out = reinterpret_cast<double*>(ctx->dcount + C_RESID);
     a.inv_perp = (T)ctx->mob.inv_perp; a.inv_par = (T)ctx->mob.inv_par;
@@ -2234,6 +2710,22 @@ static bool state_window(aLENS_ctx* ctx, const T* gg0, const T* gg1, int m, cuda
     return true;
 }
 
+// Threads of a one-barrier block of `workers` threads: a warp more for the
+// block sums and the step decision, where the block has room for it (at 1024
+// threads, or with several blocks on an SM, the last warp does both).
+static int threads1(const aLENS_ctx* ctx)
+{
+    return ctx->solve_threads <= 992 && ctx->solve_bps <= 1 ? ctx->solve_threads + 32 : ctx->solve_threads;
+}
+
+static_assert(sizeof(Shared1<double>) <= sizeof(Shared<double>) + 768 && sizeof(Shared1<float>) <= sizeof(Shared<float>) + 768,
+              "the one-barrier kernel's static shared memory and the shares' budget exceed a block's limit");
+template <typename T>
+static const void* kernel1(const aLENS_ctx* ctx)
+{
+    return threads1(ctx) <= kThreads1 ? (const void*)k_bbpgd1<T, kThreads1> : (const void*)k_bbpgd1<T, 1024>;
+}
+
 template <typename T>
 static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, int m)
 {
@@ -2283,9 +2775,9 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     // (warps 1-4 form the step decision: at least 160 threads)
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
         // one grid barrier per iteration: every block's share and its ghosts fit
-        const void* fn1 = (const void*)k_bbpgd1<T>;
+        const void* fn1 = kernel1<T>(ctx);
         const int ti = sizeof(T) == 4 ? 0 : 1;
-        const long long budget1 = (long long)optin - (long long)sizeof(Shared1<T>) - 1024;   // one block per SM
+        const long long budget1 = (long long)optin - (long long)sizeof(Shared1<T>) - 256;   // the most a block may ask for
         if (!ctx->attr1_set[ti]) {
             // the limit for the largest budget once; a launch asks for its own need
             if ((e = cudaFuncSetAttribute(fn1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget1)) !=
@@ -2297,17 +2789,21 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
         const int key = threads * 64 + bps;
         if (ctx->occ1_key[ti] != key) {
             int per_sm1 = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads, (size_t)budget)) !=
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads1(ctx), (size_t)budget)) !=
                 cudaSuccess)
                 return e;
             ctx->occ1_ok[ti] = per_sm1 >= bps;
             ctx->occ1_key[ti] = key;
         }
         if (ctx->occ1_ok[ti] && (long long)bps * ctx->num_sms >= blocks) {
+            // the share proper, with room for ds and gs (2 values for 13) and for
+            // a halo rod (6 values) per slot
+            const long long room = (long long)need1 + (long long)need1 * 8 / 13;
+            a.dyn_bytes = (size_t)(room < budget ? room : budget);
             void* args1[] = {&a};
             ++ctx->launches;
             ctx->last_solver = 1;
-            return cudaLaunchCooperativeKernel(fn1, dim3((unsigned)blocks), dim3(threads), args1, (size_t)need1,
+            return cudaLaunchCooperativeKernel(fn1, dim3((unsigned)blocks), dim3(threads1(ctx)), args1, a.dyn_bytes,
                                                ctx->stream);
         }
     }
@@ -2467,9 +2963,9 @@ static cudaError_t graph1_check(aLENS_ctx* ctx, bool& ok)
     ok = false;
     const int threads = ctx->solve_threads, bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
     if (ctx->solve_barriers != 1 || threads < 256) return cudaSuccess;
-    const void* fn1 = (const void*)k_bbpgd1<T>;
+    const void* fn1 = kernel1<T>(ctx);
     const int ti = sizeof(T) == 4 ? 0 : 1;
-    const long long budget1 = (long long)ctx->smem_optin - (long long)sizeof(Shared1<T>) - 1024;
+    const long long budget1 = (long long)ctx->smem_optin - (long long)sizeof(Shared1<T>) - 256;
     cudaError_t e;
     if (!ctx->attr1_set[ti]) {
         if ((e = cudaFuncSetAttribute(fn1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget1)) != cudaSuccess)
@@ -2477,8 +2973,8 @@ static cudaError_t graph1_check(aLENS_ctx* ctx, bool& ok)
         ctx->attr1_set[ti] = 1;
     }
     int per_sm1 = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads, (size_t)graph1_budget<T>(ctx))) !=
-        cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads1(ctx),
+                                                           (size_t)graph1_budget<T>(ctx))) != cudaSuccess)
         return e;
     ok = per_sm1 >= bps;
     return cudaSuccess;
@@ -2490,7 +2986,6 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     SolveArgs<T> a = make_args(ctx, sb, n, m);
     const bool force_redo = ctx->fault_mode == 2;   // test hook: the recorded need never fits
     ctx->fault_mode = 0;
-    const int threads = ctx->solve_threads;
     const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
     long long want = ((long long)n + 31) / 32;
     long long blocks = (long long)bps * ctx->num_sms;
@@ -2499,6 +2994,7 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     const long long budget = graph1_budget<T>(ctx);
     a.need1_dev = ctx->dcount + C_SMEM1;
     a.fit_cap = force_redo ? 0 : budget;
+    a.dyn_bytes = (size_t)budget;
     cudaError_t e;
     const int nbw = (int)blocks + 1;
     k_partition<<<(nbw * 32 + 255) / 256, 256, 0, ctx->stream>>>(n, m, (int)blocks, ctx->rowP, ctx->rowQ, ctx->bstart);
@@ -2512,8 +3008,8 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
-    return cudaLaunchCooperativeKernel((const void*)k_bbpgd1<T>, dim3((unsigned)blocks), dim3(threads), args1,
-                                       (size_t)budget, ctx->stream);
+    return cudaLaunchCooperativeKernel(kernel1<T>(ctx), dim3((unsigned)blocks), dim3(threads1(ctx)),
+                                       args1, (size_t)budget, ctx->stream);
 }
 
 cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)
