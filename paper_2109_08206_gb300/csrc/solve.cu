@@ -367,6 +367,21 @@ enum { A_STEP = 0, A_PG = 1, A_REF = 2 };
 // g = gref (delta is 0 there) and pi.pi, max |pi| at gamma_ref.
 enum { B_STEP = 0, B_REF = 2 };
 
+// g < 0 ? g : 0, and hi > lo ? hi : lo for values >= 0 (or NaN), on the
+// integer pipe: a float64 compare costs the SM's one float64 pipe 19 cycles
+// per warp, like any other float64 instruction (measured; 1e5 rods 21.4 ->
+// 20.1 ms, 2e4 rods 13.6 -> 12.8, float64).
+__device__ __forceinline__ double neg_part(double g)
+{
+    const int h = __double2hiint(g);   // (-0 stays -0; a NaN gives 0, as the compare does)
+    return h < 0 && !((h & 0x7fffffff) > 0x7ff00000 || ((h & 0x7fffffff) == 0x7ff00000 && __double2loint(g) != 0)) ? g : 0.0;
+}
+__device__ __forceinline__ double max_abs(double lo, double hi)
+{
+    const long long x = __double_as_longlong(lo), y = __double_as_longlong(hi);
+    return y > x && y <= 0x7ff0000000000000ll ? hi : lo;   // (no order with a NaN: lo stays)
+}
+
 // bil: a spring (bilateral) constraint, whose force has no sign constraint
 // (Eq. linearconstraints b): no projection.
 template <int MODE, typename T>
@@ -674,10 +689,16 @@ __device__ __forceinline__ void phase_b(const SolveArgs<T>& a, const Own<T>& o, 
         } else {
             gnew[4 * (size_t)c + 1] = gr;
         }
-        const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
+        T pi;
         // the residual is taken on the unscaled projected gradient pi / sigma_c
-        const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
-        acc[3] = api > acc[3] ? api : acc[3];
+        if constexpr (sizeof(T) == 8) {
+            pi = (bil || dm > -gam) ? gr : neg_part(gr);
+            acc[3] = max_abs(acc[3], fabs(pi) * __ldg(&a.isc[c]));
+        } else {
+            pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
+            const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
+            acc[3] = api > acc[3] ? api : acc[3];
+        }
         if (MODE == B_REF) {
             acc[0] += pi * pi;
         } else {
@@ -729,6 +750,55 @@ __device__ __forceinline__ void fold_delta(const SolveArgs<T>& a, const Own<T>& 
     }
 }
 
+// hi > lo ? hi : lo
+template <typename T>
+__device__ __forceinline__ T max_of(T lo, T hi)
+{
+    if constexpr (sizeof(T) == 8) return max_abs(lo, hi);   // (values >= 0 everywhere)
+    else return hi > lo ? hi : lo;
+}
+
+// One warp's (sum, sum, sum, max) over its lanes: lane 0, 16, 8 and 24 return
+// them.  The four values fold into one register per lane as the tree halves
+// (lanes keep one value and pass the other on), so the five levels cost six
+// exchanges and adds instead of twenty; every pair of operands is the same as in
+// a plain tree per value, and so is every bit.
+template <typename T>
+__device__ __forceinline__ T warp_sums4(const T v[4])
+{
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    // value 0 (sum) stays in lanes 0-15, value 1 (sum) in lanes 16-31; likewise 2 (sum), 3 (max)
+    const T s01 = __shfl_xor_sync(all, h16 ? v[0] : v[1], 16);
+    const T s23 = __shfl_xor_sync(all, h16 ? v[2] : v[3], 16);
+    const T a = (h16 ? v[1] : v[0]) + s01;
+    const T b = h16 ? max_of(s23, v[3]) : v[2] + s23;
+    // the maximum ends in lanes 24-31, the sums in lanes 0, 16 and 8
+    const bool is_max = h16 && h8;
+    T x = h8 ? b : a;
+    T y = __shfl_xor_sync(all, h8 ? a : b, 8);
+    x = is_max ? max_of(y, x) : x + y;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        y = __shfl_xor_sync(all, x, o);
+        const bool up = lane & o;
+        x = is_max ? max_of(up ? y : x, up ? x : y) : x + y;
+    }
+    return x;
+}
+// The value (0-3) that a lane of warp_sums4 with lane % 8 == 0 returns.
+__device__ __forceinline__ int sums4_value(int lane) { return (lane & 8 ? 2 : 0) + (lane & 16 ? 1 : 0); }
+
+// Warp w's share of the block sums into red[w].
+template <typename T>
+__device__ __forceinline__ void warp_partial(const T v[4], T (*red)[4])
+{
+    const T x = warp_sums4(v);
+    const int lane = threadIdx.x & 31;
+    if ((lane & 7) == 0) red[threadIdx.x >> 5][sums4_value(lane)] = x;
+}
+
 // Block partial of (sum, sum, sum, max) in the working precision (warp
 // shuffles, then warp 0 over the warp results, fixed order); lane 0 stores
 // it for the cross-block sum.
@@ -765,6 +835,24 @@ __device__ __forceinline__ void block_partial(T v[4], T (*red)[4], T* dst, int s
 #pragma unroll
             for (int u = 0; u < 4; ++u) dst[u * stride] = w[u];
         }
+    }
+}
+
+// The same in float64 with the folded trees: the plain ones of 24 warps are
+// 480 float64 instructions, of 19 cycles each on the SM's one float64 pipe, a
+// tenth of an iteration at 2e4 rods (solve_lcp 15.2 -> 14.3 ms).  (In float32
+// they cost nothing, and the plain trees are 1 % faster.)
+__device__ __forceinline__ void block_partial(double v[4], double (*red)[4], double* dst, int stride)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    warp_partial(v, red);
+    __syncthreads();
+    if (warp == 0) {
+        double w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = lane < nw ? red[lane][u] : 0.0;
+        const double x = warp_sums4(w);
+        if ((lane & 7) == 0) dst[sums4_value(lane) * stride] = x;
     }
 }
 
@@ -1123,8 +1211,12 @@ __global__ void k_stage_need(int nb, int esize, const int* __restrict__ bstart, 
     atomicMax(maxrods, (unsigned long long)nr);
 }
 
-template <typename T, bool ST>
-__global__ void __launch_bounds__(1024, 1) k_bbpgd(SolveArgs<T> a)
+// MAXT: the most threads of a launch (768: the default shape in float64, with
+// 80 registers a thread where 1024 leave 64 and spill: 1e5 rods 21.9 -> 21.4 ms,
+// 2e4 rods 14.3 -> 13.6; float32 does not spill and is 3 % slower with more
+// registers on the 4e5-rod pack).
+template <typename T, bool ST, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_bbpgd(SolveArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ Shared<T> sh;
@@ -1428,10 +1520,6 @@ __device__ __forceinline__ int first_item(const SolveArgs<T>& a)
 {
     return (int)threadIdx.x < a.workers ? (int)threadIdx.x : 0x40000000;
 }
-
-// hi > lo ? hi : lo
-template <typename T>
-__device__ __forceinline__ T max_of(T lo, T hi) { return hi > lo ? hi : lo; }
 
 template <typename T>
 struct Shared1 {
@@ -1956,9 +2044,15 @@ __device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1
         if (t < nc) {
             ds[t] = dm;
             gs[t] = gr;
-            const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
-            const T api = (pi < T(0) ? -pi : pi) * is;
-            acc[3] = api > acc[3] ? api : acc[3];
+            T pi;
+            if constexpr (sizeof(T) == 8) {
+                pi = (bil || dm > -gam) ? gr : neg_part(gr);
+                acc[3] = max_abs(acc[3], fabs(pi) * is);
+            } else {
+                pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
+                const T api = (pi < T(0) ? -pi : pi) * is;
+                acc[3] = api > acc[3] ? api : acc[3];
+            }
             const T sv = dm - dold, yv = gr - gold;
             acc[0] += sv * sv;
             acc[1] += sv * yv;
@@ -2082,36 +2176,6 @@ __device__ __noinline__ void fold1(const SolveArgs<T>& a, const Own1<T>& o, cons
         slot_delta(o, t) = T(0);
         if (t < o.nc) st_ref(gnew, c, hi, lo);
     }
-}
-
-// Warp w's share of the block sums: each warp's (sum, sum, sum, max) into
-// red[w].  The four values fold into one register per lane as the tree
-// halves (lanes keep one value and pass the other on), so the five levels
-// cost six exchanges instead of twenty; every pair of operands is the same
-// as in a plain tree per value, and so is every bit.
-template <typename T>
-__device__ __forceinline__ void warp_partial(const T v[4], T (*red)[4])
-{
-    const unsigned all = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const bool h16 = lane & 16, h8 = lane & 8;
-    // value 0 (sum) stays in lanes 0-15, value 1 (sum) in lanes 16-31; likewise 2 (sum), 3 (max)
-    const T s01 = __shfl_xor_sync(all, h16 ? v[0] : v[1], 16);
-    const T s23 = __shfl_xor_sync(all, h16 ? v[2] : v[3], 16);
-    const T a = (h16 ? v[1] : v[0]) + s01;
-    const T b = h16 ? max_of(s23, v[3]) : v[2] + s23;
-    // the maximum ends in lanes 24-31, the sums in lanes 0, 16 and 8
-    const bool is_max = h16 && h8;
-    T x = h8 ? b : a;
-    T y = __shfl_xor_sync(all, h8 ? a : b, 8);
-    x = is_max ? max_of(y, x) : x + y;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        y = __shfl_xor_sync(all, x, o);
-        const bool up = lane & o;
-        x = is_max ? max_of(up ? y : x, up ? x : y) : x + y;
-    }
-    if ((lane & 7) == 0) red[threadIdx.x >> 5][h8 ? (h16 ? 3 : 2) : (h16 ? 1 : 0)] = x;
 }
 
 // One warp after a block barrier: the block's sums over the workers' red;
@@ -2815,7 +2879,9 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     a.sort_ns = sizeof(T) == 8 && !staged && maxrods > 0 && maxrods < 65536 && sort_bytes <= budget;
     a.sort_cap = (int)maxrods;
     const size_t smem = staged ? (size_t)need : (a.sort_ns ? (size_t)sort_bytes : 0);
-    const void* fn = staged ? (const void*)k_bbpgd<T, true> : (const void*)k_bbpgd<T, false>;
+    constexpr int kMaxT = sizeof(T) == 8 ? 768 : 1024;
+    const void* fn = threads <= kMaxT ? (staged ? (const void*)k_bbpgd<T, true, kMaxT> : (const void*)k_bbpgd<T, false, kMaxT>)
+                                      : (staged ? (const void*)k_bbpgd<T, true, 1024> : (const void*)k_bbpgd<T, false, 1024>);
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     int per_sm = 0;
