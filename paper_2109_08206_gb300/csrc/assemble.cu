@@ -575,17 +575,14 @@ cudaError_t launch_solve_layout(aLENS_ctx* ctx, int n, int m, const int32_t* pai
 {
     cudaStream_t st = ctx->stream;
     cudaError_t e;
-    size_t bytes = sizeof(int) * ((size_t)n + 1);
-    if ((e = cudaMemsetAsync(ctx->rod_count, 0, bytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ctx->cntQ, 0, bytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ctx->curQ, 0, bytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ctx->curP, 0, bytes, st)) != cudaSuccess) return e;
+    int* const counts[4] = {ctx->rod_count, ctx->cntQ, ctx->curQ, ctx->curP};
+    const int lens[4] = {n + 1, n + 1, n + 1, n + 1};
+    if ((e = zero_ints(ctx, 4, counts, lens)) != cudaSuccess) return e;
     if (m > 0) {
         k_count_sides<<<nblk(m, 256), 256, 0, st>>>(m, pairs, rank, ctx->rod_count, ctx->cntQ, ctx->mdev);
         ++ctx->launches;
     }
-    if ((e = exclusive_scan(ctx, ctx->rod_count, ctx->rowP, n)) != cudaSuccess) return e;
-    if ((e = exclusive_scan(ctx, ctx->cntQ, ctx->rowQ, n)) != cudaSuccess) return e;
+    if ((e = exclusive_scan2(ctx, ctx->rod_count, ctx->rowP, ctx->cntQ, ctx->rowQ, n)) != cudaSuccess) return e;
     if (m > 0) {
         k_scatter_owner<<<nblk(m, 256), 256, 0, st>>>(m, pairs, rank, ctx->rowP, ctx->curP, ctx->perm, ctx->mdev);
         ++ctx->launches;

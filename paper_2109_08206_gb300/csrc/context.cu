@@ -208,7 +208,7 @@ aLENS_status grow_keys(aLENS_ctx* c, long long nkeys)
     CK(cudaStreamSynchronize(c->stream));
     int* na[3] = {nullptr, nullptr, nullptr};
     int* nscan = nullptr;
-    int tiles = (int)((std::max((long long)c->max_rods, nkeys) + 4095) / 4096) + 2;
+    int tiles = (int)((std::max(2 * (long long)c->max_rods, nkeys) + 4095) / 4096) + 3;
     bool ok = true;
     for (int k = 0; k < 3; ++k) ok &= dmalloc(&na[k], ((size_t)nkeys + 1) * sizeof(int)) == cudaSuccess;
     if (tiles > c->scan_tmp_len) ok &= dmalloc(&nscan, (size_t)tiles * sizeof(int)) == cudaSuccess;
@@ -389,7 +389,7 @@ aLENS_status aLENS_create(const aLENS_params* params, int64_t max_rods, int64_t 
     c->max_keys = 1 << (3 * geo.bits);
     c->max_blocks = c->num_sms * 8;
     size_t np = (size_t)max_rods, mp = (size_t)max_pairs;
-    int scan_tiles = (int)((std::max(np, (size_t)c->max_keys) + 4095) / 4096) + 2;
+    int scan_tiles = (int)((std::max(2 * np, (size_t)c->max_keys) + 4095) / 4096) + 3;   // (two arrays of np at once)
     c->scan_tmp_len = scan_tiles;
     bool ok = true;
     ok &= dmalloc(&c->xw, 3 * np * sizeof(double)) == cudaSuccess;
@@ -584,14 +584,12 @@ static aLENS_status search_kernels(aLENS_ctx* c, int n, const double* x, const d
     int nkeys = c->cur_nkeys;
     aLENS_status st = reset_status(c);
     if (st != ALENS_OK) return st;
-    CK(cudaMemsetAsync(c->cell_count, 0, ((size_t)nkeys + 1) * sizeof(int), c->stream));
-    CK(cudaMemsetAsync(c->cell_cursor, 0, ((size_t)nkeys + 1) * sizeof(int), c->stream));
-    CK(cudaMemsetAsync(c->rod_count, 0, ((size_t)n + 1) * sizeof(int), c->stream));
+    const bool walls = c->wall_axis >= 0 && c->cur_systab == nullptr;
+    int* const counts[4] = {c->cell_count, c->cell_cursor, c->rod_count, c->cntQ};
+    const int lens[4] = {nkeys + 1, nkeys + 1, n + 1, n + 1};
+    CK(zero_ints(c, walls ? 4 : 3, counts, lens));
     CK(launch_pack(c, n, x, quat, fnc, true));
-    if (c->wall_axis >= 0 && c->cur_systab == nullptr) {
-        CK(cudaMemsetAsync(c->cntQ, 0, ((size_t)n + 1) * sizeof(int), c->stream));
-        CK(launch_count_walls(c, n));
-    }
+    if (walls) CK(launch_count_walls(c, n));
     CK(launch_cell_sort(c, n));
     CK(launch_search(c, n));
     return ALENS_OK;
@@ -737,7 +735,6 @@ static aLENS_status fork_layout(aLENS_ctx* c, int n, int m, const double* quat)
     CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     {
         StreamSwap on(c, c->side);
-        CK(launch_rank(c, n));
         CK(launch_solve_layout(c, n, m, c->pairs, quat, c->p.precision, c->rank));
     }
     CK(cudaEventRecord(c->ev_join, c->side));
@@ -787,7 +784,6 @@ static aLENS_status step_impl(aLENS_ctx* c, int64_t n, double* x, double* quat, 
     if (beside) {
         CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
     } else {
-        CK(launch_rank(c, (int)n));
         CK(launch_solve_layout(c, (int)n, (int)m, c->pairs, quat, c->p.precision, c->rank));
     }
     CK(launch_solve_fill(c, (int)n, (int)m, c->pairs, c->dgeom, c->q64, gin, c->p.precision, c->rank));

@@ -461,6 +461,10 @@ namespace alens {
 
 // scan.cu: exclusive scan of counts[0..n) into out[0..n], out[n] = total.
 cudaError_t exclusive_scan(aLENS_ctx* ctx, const int* counts, int* out, int n);
+// Two arrays of the same length at once.
+cudaError_t exclusive_scan2(aLENS_ctx* ctx, const int* counts0, int* out0, const int* counts1, int* out1, int n);
+// Zeroes up to four int arrays in one launch.
+cudaError_t zero_ints(aLENS_ctx* ctx, int arrays, int* const* p, const int* n);
 
 // neighbors.cu
 cudaError_t launch_pack(aLENS_ctx* ctx, int n, const double* x, const double* quat, const double* fnc, bool cells);
@@ -491,8 +495,6 @@ cudaError_t launch_solve_fill(aLENS_ctx* ctx, int n, int m, const int32_t* pairs
 cudaError_t launch_solve_setup(aLENS_ctx* ctx, int n, int m, const int32_t* pairs, const double* dgeom,
                                const double* q, const double* gamma_in, const double* quat, int precision,
                                const int* rank);
-// rank[sorted_id[k]] = k: the cell-sorted position of every rod.
-cudaError_t launch_rank(aLENS_ctx* ctx, int n);
 
 // solve.cu
 cudaError_t launch_solve(aLENS_ctx* ctx, int n, int m, int precision);

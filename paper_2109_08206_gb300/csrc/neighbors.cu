@@ -149,13 +149,15 @@ k_cell_sort_ids(int nkeys, const int* __restrict__ cell_start, int* __restrict__
 }
 
 __global__ void k_cell_gather(int n, const int* __restrict__ sorted_id, const float4* __restrict__ pos32,
-                              const float4* __restrict__ ax32, float4* __restrict__ spos32, float4* __restrict__ sax32)
+                              const float4* __restrict__ ax32, float4* __restrict__ spos32, float4* __restrict__ sax32,
+                              int* __restrict__ rank)
 {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     int i = sorted_id[k];
     spos32[k] = pos32[i];
     sax32[k] = ax32[i];
+    rank[i] = k;   // the solver's position of the rod
 }
 
 // Float32 screen of one candidate: kScreenDrop when the pair is certainly
@@ -560,7 +562,7 @@ cudaError_t launch_cell_sort(aLENS_ctx* ctx, int n)
                                                                                        ctx->sorted_id);
         ++ctx->launches;
         k_cell_gather<<<nblk(n, 256), 256, 0, ctx->stream>>>(n, ctx->sorted_id, ctx->pos32, ctx->ax32, ctx->spos32,
-                                                             ctx->sax32);
+                                                             ctx->sax32, ctx->rank);
         ++ctx->launches;
     }
     return cudaGetLastError();

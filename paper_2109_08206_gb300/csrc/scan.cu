@@ -1,7 +1,12 @@
-// Exclusive prefix sum of int32 counts (CSR row pointers, cell starts).
-// Two launches: per-tile totals, then per-tile scans, each block adding the
-// totals of the tiles before it (a few thousand at most) for its offset.
-// Integer sums: exact and deterministic.
+// Exclusive prefix sums of int32 counts (CSR row pointers, cell starts), one
+// array or two of the same length at once (grid.y), and the zeroing of count
+// arrays.  Small steps are bound by their launches (about 3 us each, most of
+// it the launch): a single-system step
+// had 11 memsets and 30 kernels.
+// Up to kScanSmall entries one block scans an array tile after tile (1.6e4
+// entries: 4 us; two launches 6 to 9).  More: per-tile totals, then per-tile
+// scans, each block adding the totals of the tiles before it (a few thousand at
+// most) for its offset.  Integer sums: exact and deterministic.
 #include "internal.cuh"
 
 namespace alens {
@@ -40,9 +45,44 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* smem, int& total
     return r;
 }
 
-__global__ void k_tile_sums(const int* __restrict__ in, int n, int* __restrict__ sums)
+constexpr int kScanSmall = 4 * kScanTile;
+
+struct ScanArrays {
+    const int* in[2];
+    int* out[2];
+};
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_small(ScanArrays s, int n)
 {
     __shared__ int smem[64];
+    const int* __restrict__ in = s.in[blockIdx.x];
+    int* __restrict__ out = s.out[blockIdx.x];
+    int before = 0;
+    for (int t = 0; t < n; t += kScanTile) {
+        const int base = t + (int)threadIdx.x * kScanItems;
+        int v[kScanItems], acc = 0;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            v[k] = base + k < n ? in[base + k] : 0;
+            acc += v[k];
+        }
+        int total;
+        int ex = block_exclusive_scan(acc, smem, total) + before;
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            if (base + k < n) out[base + k] = ex;
+            ex += v[k];
+        }
+        before += total;
+    }
+    if (threadIdx.x == 0) out[n] = before;
+}
+
+// sums: [arrays][gridDim.x] tile totals
+__global__ void k_tile_sums(ScanArrays s, int n, int* __restrict__ sums)
+{
+    __shared__ int smem[64];
+    const int* __restrict__ in = s.in[blockIdx.y];
     long long base = (long long)blockIdx.x * kScanTile;
     int acc = 0;
     for (int k = 0; k < kScanItems; ++k) {
@@ -51,16 +91,18 @@ __global__ void k_tile_sums(const int* __restrict__ in, int n, int* __restrict__
     }
     int total;
     block_exclusive_scan(acc, smem, total);
-    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+    if (threadIdx.x == 0) sums[blockIdx.y * gridDim.x + blockIdx.x] = total;
 }
 
-__global__ void k_tile_scan(const int* __restrict__ in, int n, const int* __restrict__ sums, int* __restrict__ out)
+__global__ void k_tile_scan(ScanArrays s, int n, const int* __restrict__ sums)
 {
     __shared__ int smem[64];
     __shared__ int pre;
+    const int* __restrict__ in = s.in[blockIdx.y];
+    int* __restrict__ out = s.out[blockIdx.y];
     if (threadIdx.x < 32) {   // this tile's offset: the totals of the tiles before it
         int a = 0;
-        for (int t = threadIdx.x; t < (int)blockIdx.x; t += 32) a += sums[t];
+        for (int t = threadIdx.x; t < (int)blockIdx.x; t += 32) a += sums[blockIdx.y * gridDim.x + t];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
         if (threadIdx.x == 0) pre = a;
@@ -86,13 +128,54 @@ __global__ void k_tile_scan(const int* __restrict__ in, int n, const int* __rest
 
 // k_tile_sums sums a tile in strided order and k_tile_scan scans it in
 // blocked order; both cover the same kScanTile elements, so the tile totals agree.
+static cudaError_t scan_arrays(aLENS_ctx* ctx, const ScanArrays& s, int arrays, int n)
+{
+    if (n <= kScanSmall) {
+        k_scan_small<<<arrays, kScanThreads, 0, ctx->stream>>>(s, n);
+        ++ctx->launches;
+        return cudaGetLastError();
+    }
+    const int ntiles = (n + kScanTile - 1) / kScanTile;
+    if (arrays * ntiles > ctx->scan_tmp_len) return cudaErrorInvalidValue;
+    k_tile_sums<<<dim3(ntiles, arrays), kScanThreads, 0, ctx->stream>>>(s, n, ctx->scan_tmp);
+    ++ctx->launches;
+    k_tile_scan<<<dim3(ntiles, arrays), kScanThreads, 0, ctx->stream>>>(s, n, ctx->scan_tmp);
+    ++ctx->launches;
+    return cudaGetLastError();
+}
+
 cudaError_t exclusive_scan(aLENS_ctx* ctx, const int* counts, int* out, int n)
 {
-    int ntiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
-    if (ntiles + 1 > ctx->scan_tmp_len) return cudaErrorInvalidValue;
-    k_tile_sums<<<ntiles, kScanThreads, 0, ctx->stream>>>(counts, n, ctx->scan_tmp);
-    ++ctx->launches;
-    k_tile_scan<<<ntiles, kScanThreads, 0, ctx->stream>>>(counts, n, ctx->scan_tmp, out);
+    return scan_arrays(ctx, ScanArrays{{counts, nullptr}, {out, nullptr}}, 1, n);
+}
+
+cudaError_t exclusive_scan2(aLENS_ctx* ctx, const int* counts0, int* out0, const int* counts1, int* out1, int n)
+{
+    return scan_arrays(ctx, ScanArrays{{counts0, counts1}, {out0, out1}}, 2, n);
+}
+
+struct ZeroArrays {
+    int* p[4];
+    int n[4];
+};
+
+__global__ void k_zero_ints(ZeroArrays z)
+{
+    int* const p = z.p[blockIdx.y];
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < z.n[blockIdx.y]; k += gridDim.x * blockDim.x) p[k] = 0;
+}
+
+cudaError_t zero_ints(aLENS_ctx* ctx, int arrays, int* const* p, const int* n)
+{
+    ZeroArrays z = {};
+    int most = 1;
+    for (int k = 0; k < arrays; ++k) {
+        z.p[k] = p[k];
+        z.n[k] = n[k];
+        if (n[k] > most) most = n[k];
+    }
+    const int blocks = (most + 1023) / 1024;
+    k_zero_ints<<<dim3(blocks < 1024 ? blocks : 1024, arrays), 256, 0, ctx->stream>>>(z);
     ++ctx->launches;
     return cudaGetLastError();
 }

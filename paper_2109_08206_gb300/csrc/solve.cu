@@ -754,7 +754,7 @@ __device__ __forceinline__ void fold_delta(const SolveArgs<T>& a, const Own<T>& 
 template <typename T>
 __device__ __forceinline__ T max_of(T lo, T hi)
 {
-    if constexpr (sizeof(T) == 8) return max_abs(lo, hi);   // (values >= 0 everywhere)
+    if constexpr (sizeof(T) == 8) return max_abs(lo, hi);   // (magnitudes everywhere: values >= 0)
     else return hi > lo ? hi : lo;
 }
 
@@ -1183,32 +1183,6 @@ __device__ __forceinline__ void solve_loop(const SolveArgs<T>& a, const Own<T>& 
     }
     if (threadIdx.x == 0) sh.cur = st.cur;
     __syncthreads();
-}
-
-// One warp per block boundary b in [0, nb]: the work-balanced split.
-__global__ void k_partition(int n, int m, int nb, const int* __restrict__ rowP, const int* __restrict__ rowQ,
-                            int* __restrict__ bstart)
-{
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (b > nb) return;   // uniform per warp
-    const long long total = rank_work(rowP, rowQ, n);
-    const int r = b == nb ? n : find_rank(rowP, rowQ, 0, n, total * b / nb);
-    if ((threadIdx.x & 31) == 0) bstart[b] = r;
-}
-
-// Largest shared-memory share over the blocks (bytes, for element size esize)
-// and the largest rod count of a block.
-__global__ void k_stage_need(int nb, int esize, const int* __restrict__ bstart, const int* __restrict__ rowP,
-                             const int* __restrict__ rowQ, unsigned long long* __restrict__ need,
-                             unsigned long long* __restrict__ maxrods)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nb) return;
-    const int r0 = bstart[b], r1 = bstart[b + 1];
-    const size_t nc = rowP[r1] - rowP[r0], nq = rowQ[r1] - rowQ[r0], nr = r1 - r0;
-    const size_t bytes = staged_bytes(esize, nc, nr, nq);
-    atomicMax(need, (unsigned long long)bytes);
-    atomicMax(maxrods, (unsigned long long)nr);
 }
 
 // MAXT: the most threads of a launch (768: the default shape in float64, with
@@ -2458,19 +2432,34 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
     }
 }
 
-// One thread block per solver block b (kNeedThreads threads): the
-// one-barrier kernel's shared-memory share (ghosts counted from the block's
-// other-side entries); a share whose slot or rod count exceeds the 15-bit
-// local indices does not fit.
+// The work-balanced split and what its shares need, one thread block per solver block b
+// in one launch (three before): the share's two boundaries (bstart; a warp
+// each), the two-barrier kernel's largest shared-memory share and rod count
+// over the blocks (need, maxrods), and the one-barrier kernel's (need1; ghosts
+// counted from the block's other-side entries; a share whose slot or rod
+// count exceeds the 15-bit local indices does not fit).  Also zeroes the
+// solver's barrier words.  The three counters are zero before (reset with the step's).
 constexpr int kNeedThreads = 256;
 __global__ void __launch_bounds__(kNeedThreads)
-k_stage_need1(int nb, int esize, const int* __restrict__ bstart, const int* __restrict__ rowP,
-              const int* __restrict__ rowQ, const int* __restrict__ qlist, unsigned long long* __restrict__ need)
+k_shares(int n, int nb, int esize, const int* __restrict__ rowP, const int* __restrict__ rowQ,
+         const int* __restrict__ qlist, int* __restrict__ bstart, unsigned* __restrict__ bar,
+         unsigned long long* __restrict__ need, unsigned long long* __restrict__ maxrods,
+         unsigned long long* __restrict__ need1)
 {
-    __shared__ int wsum[kNeedThreads / 32];
+    __shared__ int wsum[kNeedThreads / 32], bound[2];
     const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (b >= nb) return;   // uniform per block
-    const int r0 = bstart[b], r1 = bstart[b + 1];
+    if (warp < 2) {
+        const int k = b + warp;
+        const long long total = rank_work(rowP, rowQ, n);
+        const int r = k == nb ? n : find_rank(rowP, rowQ, 0, n, total * k / nb);
+        if (lane == 0) {
+            bound[warp] = r;
+            if (warp == 0 || k == nb) bstart[k] = r;
+        }
+    }
+    if (b == 0 && threadIdx.x < 4) bar[threadIdx.x] = 0u;
+    __syncthreads();
+    const int r0 = bound[0], r1 = bound[1];
     const int c0 = rowP[r0], c1 = rowP[r1], q0 = rowQ[r0], q1 = rowQ[r1];
     int ng = 0;
     for (int k = q0 + (int)threadIdx.x; k < q1; k += kNeedThreads) {
@@ -2484,10 +2473,12 @@ k_stage_need1(int nb, int esize, const int* __restrict__ bstart, const int* __re
     if (threadIdx.x == 0) {
         ng = 0;
         for (int w = 0; w < kNeedThreads / 32; ++w) ng += wsum[w];
-        const size_t nt = (size_t)(c1 - c0) + ng, nr = r1 - r0;
-        unsigned long long bytes = staged1_bytes(esize, nt, ng, nr, q1 - q0, nb);
+        const size_t nc = (size_t)(c1 - c0), nt = nc + ng, nr = r1 - r0, nq = q1 - q0;
+        atomicMax(need, (unsigned long long)staged_bytes(esize, nc, nr, nq));
+        atomicMax(maxrods, (unsigned long long)nr);
+        unsigned long long bytes = staged1_bytes(esize, nt, ng, nr, nq, nb);
         if (nt > (size_t)kMaxSlots || nr > (size_t)kMaxSlots) bytes = ~0ull;
-        atomicMax(need, bytes);
+        atomicMax(need1, bytes);
     }
 }
 
@@ -2654,20 +2645,6 @@ __global__ void k_gamma_out(int m, const int* __restrict__ flags, const int* __r
     out[perm[c]] = scale64[c] * (((double)g[4 * (size_t)c + 2] + (double)g[4 * (size_t)c + 3]) + (double)g[4 * (size_t)c]);
 }
 
-__global__ void k_rank(int n, const int* __restrict__ sorted_id, int* __restrict__ rank)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) rank[sorted_id[k]] = k;
-}
-
-cudaError_t launch_rank(aLENS_ctx* ctx, int n)
-{
-    if (n <= 0) return cudaSuccess;
-    k_rank<<<(n + 255) / 256, 256, 0, ctx->stream>>>(n, ctx->sorted_id, ctx->rank);
-    ++ctx->launches;
-    return cudaGetLastError();
-}
-
 // Largest value f of type T with hD * (double)f <= tol in float64 (the
 // float64 product is monotone in f, so max |pi| <= f exactly when the float64
 // residual test passes); -1 when no f >= 0 passes.
@@ -2807,23 +2784,11 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     // work-balanced split, then the largest shared-memory share: stage every
     // block's data when all shares fit the opt-in budget (one readback)
     cudaError_t e;
-    const int nbw = (int)blocks + 1;
-    k_partition<<<(nbw * 32 + 255) / 256, 256, 0, ctx->stream>>>(n, m, (int)blocks, ctx->rowP, ctx->rowQ, ctx->bstart);
+    k_shares<<<(int)blocks, kNeedThreads, 0, ctx->stream>>>(n, (int)blocks, (int)sizeof(T), ctx->rowP, ctx->rowQ, ctx->qlist,
+                                                             ctx->bstart, ctx->bar, ctx->dcount + C_SMEM,
+                                                             ctx->dcount + C_MAXRODS, ctx->dcount + C_SMEM1);
     ++ctx->launches;
-    // counters C_SMEM, and C_MAXRODS and C_SMEM1 (adjacent)
-    if ((e = cudaMemsetAsync(ctx->dcount + C_SMEM, 0, sizeof(unsigned long long), ctx->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(ctx->dcount + C_MAXRODS, 0, 2 * sizeof(unsigned long long), ctx->stream)) != cudaSuccess)
-        return e;
-    k_stage_need<<<((int)blocks + 127) / 128, 128, 0, ctx->stream>>>((int)blocks, (int)sizeof(T), ctx->bstart, ctx->rowP,
-                                                                  ctx->rowQ, ctx->dcount + C_SMEM,
-                                                                  ctx->dcount + C_MAXRODS);
-    ++ctx->launches;
-    if (ctx->solve_barriers == 1) {
-        k_stage_need1<<<(int)blocks, kNeedThreads, 0, ctx->stream>>>((int)blocks, (int)sizeof(T), ctx->bstart,
-                                                                      ctx->rowP, ctx->rowQ, ctx->qlist,
-                                                                      ctx->dcount + C_SMEM1);
-        ++ctx->launches;
-    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // one readback of the counters C_SMEM .. C_SMEM1 (into the pinned host status
     // buffer; the allocation-free entry point has none and reads into the stack)
     unsigned long long local[C_SMEM1 - C_SMEM + 1];
@@ -2835,8 +2800,6 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     const unsigned long long need = hb[0], maxrods = hb[C_MAXRODS - C_SMEM], need1 = hb[C_SMEM1 - C_SMEM];
     const int optin = ctx->smem_optin;
     const long long budget = (long long)optin / bps - (long long)sizeof(Shared<T>) - 1024;
-    if ((e = cudaMemsetAsync(ctx->bar, 0, 4 * sizeof(unsigned), ctx->stream)) != cudaSuccess) return e;
-    // (warps 1-4 form the step decision: at least 160 threads)
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
         // one grid barrier per iteration: every block's share and its ghosts fit
         const void* fn1 = kernel1<T>(ctx);
@@ -3011,7 +2974,7 @@ cudaError_t launch_solve(aLENS_ctx* ctx, int n, int m, int precision)
 // The single-system solve of a step recorded as a CUDA graph: no readback.
 // The one-barrier kernel is launched with the full shared-memory budget of
 // the launch shape, and its blocks check the need of the shares (computed
-// on the device by k_stage_need1) against it: a share that does not fit
+// on the device by k_shares) against it: a share that does not fit
 // makes every block leave before its first barrier with kSolveRedo in
 // F_SOLVE_ERR, the update and the outputs then leave everything untouched,
 // and the caller runs the step eagerly.  graph1_possible says whether the
@@ -3062,15 +3025,11 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     a.fit_cap = force_redo ? 0 : budget;
     a.dyn_bytes = (size_t)budget;
     cudaError_t e;
-    const int nbw = (int)blocks + 1;
-    k_partition<<<(nbw * 32 + 255) / 256, 256, 0, ctx->stream>>>(n, m, (int)blocks, ctx->rowP, ctx->rowQ, ctx->bstart);
+    k_shares<<<(int)blocks, kNeedThreads, 0, ctx->stream>>>(n, (int)blocks, (int)sizeof(T), ctx->rowP, ctx->rowQ, ctx->qlist,
+                                                             ctx->bstart, ctx->bar, ctx->dcount + C_SMEM,
+                                                             ctx->dcount + C_MAXRODS, ctx->dcount + C_SMEM1);
     ++ctx->launches;
-    if ((e = cudaMemsetAsync(ctx->dcount + C_SMEM1, 0, sizeof(unsigned long long), ctx->stream)) != cudaSuccess) return e;
-    k_stage_need1<<<(int)blocks, kNeedThreads, 0, ctx->stream>>>((int)blocks, (int)sizeof(T), ctx->bstart,
-                                                                  ctx->rowP, ctx->rowQ, ctx->qlist,
-                                                                  ctx->dcount + C_SMEM1);
-    ++ctx->launches;
-    if ((e = cudaMemsetAsync(ctx->bar, 0, 4 * sizeof(unsigned), ctx->stream)) != cudaSuccess) return e;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
