@@ -575,6 +575,7 @@ cudaError_t launch_solve_layout(aLENS_ctx* ctx, int n, int m, const int32_t* pai
 {
     cudaStream_t st = ctx->stream;
     cudaError_t e;
+    ctx->caller_order = rank == nullptr;
     int* const counts[4] = {ctx->rod_count, ctx->cntQ, ctx->curQ, ctx->curP};
     const int lens[4] = {n + 1, n + 1, n + 1, n + 1};
     if ((e = zero_ints(ctx, 4, counts, lens)) != cudaSuccess) return e;

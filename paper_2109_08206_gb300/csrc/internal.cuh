@@ -382,11 +382,12 @@ struct aLENS_ctx {
     size_t persist_prev;     // the context's persisting set-aside before this context raised it
     size_t persist_set;      // the set-aside this context set (0: untouched)
     int l2_window_off;       // aLENS_set_l2_window(ctx, 0)
-    int attr1_set[2];        // the one-barrier kernel's dynamic shared-memory limit is set (float, double)
-    int occ1_key[2];         // launch shape (threads * 64 + blocks per SM) whose occupancy was checked ...
+    int attr1_set[2];        // the one-barrier kernels' dynamic shared-memory limits that are set (a bit each; float, double)
+    int occ1_key[2];         // kernel and launch shape whose occupancy was checked ...
     int occ1_ok[2];          // ... and whether that many blocks per SM fit at the full budget
     int last_solver;         // kernel of the last single-system solve: 1 one-barrier, 2 two-barrier staged, 3 two-barrier global
     int zero_start;          // the last setup started from gamma = 0 (no caller gamma)
+    int caller_order;        // the last layout took the rods in the caller's order (no rank)
     int qe_pending;          // the last setup's CSR-ordered other-side copies (qe) are still to be written
     int qe_m, qe_prec;       // ... for this many constraints in this precision
     // batched steps as a captured CUDA graph (aLENS_set_batch_graph)

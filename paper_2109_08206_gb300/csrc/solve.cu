@@ -1284,8 +1284,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd(SolveArgs<T> a)
 // ms a step, 5e3 rods 0.86 -> 0.66, 2e4 rods 1.98 -> 1.45, 5e4 rods 1.43 ->
 // 1.25, 1e5 rods 3.90 -> 3.60 (366 iterations), 1e4 rods float64 2.17 -> 1.56.
 // Where the rods come in no spatial order (a large solve_lcp) nearly every
-// slot's other end is in the halo and the polls cost more than they save: 5e4
-// rods 2.08 -> 2.50.
+// slot's other end is in the halo and the polls cost more than they save: those
+// keep the barrier (k_bbpgd1_meet).
 
 // A block's share: rods [r0, r1), owned constraints [c0, c1) in slots
 // [0, nc), ghosts in slots [nc, nt).
@@ -2432,6 +2432,710 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
     }
 }
 
+// ---------------------------------------------------------------------
+// The same iteration with one grid barrier, for large systems whose rods come
+// in no spatial order (solve_lcp takes the caller's order): nearly every
+// slot's other end then lies in another block, and the halo of tagged words
+// costs more to poll than a barrier and plain gathers of the slots' own words
+// (solve, barrier / tagged: 3e4 rods 0.65 / 0.84 ms, 5e4 rods 2.10 / 2.48;
+// 8e3 rods 0.71 / 0.56, so the line lies between).  One thread per rod, a
+// slot's values in columns; the sums are the same in the same order, and so
+// is every bit.
+constexpr int kMeetRods = 16000;
+namespace meet {
+
+constexpr unsigned kBil = 0x8000u;   // bilateral (spring) constraint: no projection
+constexpr int kLocal = 0x7fff;
+
+// A block's share: rods [r0, r1), owned constraints [c0, c1) in slots
+// [0, nc), ghosts in slots [nc, nt).
+template <typename T>
+struct Own1 {
+    int r0, r1, c0, c1, q0, q1, nc, ng, nt, cap_r, nbp;
+    T* tot;      // [4][nbp] last barrier's block sums (cp.async target)
+    T* rec;      // [9][nt]
+    T* gref;     // [nt] q + D^T Uref
+    T* ds;       // [nt] delta
+    T* grs;      // [nt] g
+    T* gam;      // [nt] gamma_ref
+    T* ax;       // [3][cap_r]
+    T* U;        // [6][cap_r] this iteration's dU (the reference velocity during a refresh)
+    int* oth;    // [nt] rank of the slot's other end: Q for owned slots, the owner for ghosts (-1: a wall)
+    int* gid;    // [ng] constraint id of ghost slot nc + g
+    int* rowP;   // [cap_r + 1] owned ranges (constraint ids; slot = id - c0)
+    int* rowQ;   // [cap_r + 1] other-side ranges (CSR positions)
+    unsigned short* loc;    // [nt] local index of the slot's rod in this block (P owned, Q ghost), | kBil
+    unsigned short* qslot;  // [q1 - q0] slot of each other-side entry, | kBil
+    unsigned short* perm;   // [cap_r] rod order of the rod phase
+};
+template <typename T>
+__device__ void carve1(Own1<T>& o, unsigned char* base)
+{
+    const size_t nt = o.nt, R = o.cap_r;
+    o.tot = reinterpret_cast<T*>(base);
+    base += align16(4 * (size_t)o.nbp * sizeof(T));
+    T* t = reinterpret_cast<T*>(base);
+    o.rec = t; t += 9 * nt;
+    o.gref = t; t += nt;
+    o.ds = t; t += nt;
+    o.grs = t; t += nt;
+    o.gam = t; t += nt;
+    o.ax = t; t += 3 * R;
+    o.U = t; t += 6 * R;
+    base += align16((13 * nt + 9 * R) * sizeof(T));
+    int* ip = reinterpret_cast<int*>(base);
+    o.oth = ip; ip += nt;
+    o.gid = ip; ip += o.ng;
+    o.rowP = ip; ip += R + 1;
+    o.rowQ = ip; ip += R + 1;
+    base += align16((nt + o.ng + 2 * R + 2) * sizeof(int));
+    unsigned short* sp = reinterpret_cast<unsigned short*>(base);
+    o.loc = sp; sp += nt;
+    o.qslot = sp; sp += o.q1 - o.q0;
+    o.perm = sp;
+}
+
+template <typename T>
+struct Shared1 {
+    T red[32][4];
+    T tot[4];   // grid totals of the last barrier's block sums (warps 1-4, one each)
+    T alpha;
+    int kind, ng;
+};
+
+// Stage one slot (owned or ghost) of constraint c from the global arrays.
+template <typename T>
+__device__ __forceinline__ void stage_slot(const SolveArgs<T>& a, const Own1<T>& o, int t, int c, int li, int other,
+                                           unsigned bil)
+{
+    const size_t mp = a.mp, nt = o.nt;
+#pragma unroll
+    for (int w = 0; w < 9; ++w) o.rec[w * nt + t] = a.rec[w * mp + c];
+    T d, g, gr, gl;
+    ld_state(a.gg0, c, d, g, gr, gl);
+    o.ds[t] = d;
+    o.gam[t] = gr;
+    o.grs[t] = gl;   // gamma_lo until the first reference pass replaces it by g
+    o.gref[t] = T(0);
+    o.oth[t] = other;
+    o.loc[t] = (unsigned short)(li | bil);
+}
+
+template <typename T>
+__device__ void stage_in1(const SolveArgs<T>& a, Own1<T>& o, unsigned char* dyn, Shared1<T>& sh)
+{
+    const int nr = o.r1 - o.r0, nq = o.q1 - o.q0;
+    // ghosts: other-side entries of the block's rods that another block owns
+    if (threadIdx.x == 0) sh.ng = 0;
+    __syncthreads();
+    int cnt = 0;
+    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+        const int c = a.qlist[o.q0 + k];
+        cnt += c < o.c0 || c >= o.c1;
+    }
+    if (cnt) atomicAdd(&sh.ng, cnt);
+    __syncthreads();
+    o.ng = sh.ng;
+    o.nt = o.nc + o.ng;
+    carve1(o, dyn);
+    __syncthreads();
+    if (threadIdx.x == 0) sh.ng = 0;
+    for (int li = threadIdx.x; li <= nr; li += blockDim.x) {
+        o.rowP[li] = a.rowP[o.r0 + li];
+        o.rowQ[li] = a.rowQ[o.r0 + li];
+    }
+    for (int li = threadIdx.x; li < nr; li += blockDim.x)
+        for (int w = 0; w < 3; ++w) o.ax[w * o.cap_r + li] = a.ax[w * (size_t)a.np + o.r0 + li];
+    const bool has_comp = a.comp != nullptr;
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) {
+        const int c = o.c0 + t;
+        const unsigned bil = has_comp && a.comp[c] >= T(0) ? kBil : 0u;
+        stage_slot(a, o, t, c, a.ci[c] - o.r0, a.cj[c], bil);
+    }
+    __syncthreads();   // sh.ng is 0 again before the slots are numbered
+#pragma unroll 1
+    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+        const int c = a.qlist[o.q0 + k];
+        const unsigned bil = has_comp && a.comp[c] >= T(0) ? kBil : 0u;
+        int t;
+        if (c < o.c0 || c >= o.c1) {
+            // the slot order of ghosts does not enter any result
+            const int g = atomicAdd(&sh.ng, 1);
+            t = o.nc + g;
+            o.gid[g] = c;
+            stage_slot(a, o, t, c, a.cj[c] - o.r0, a.ci[c], bil);
+        } else {
+            t = c - o.c0;
+        }
+        o.qslot[k] = (unsigned short)(t | bil);
+    }
+    __syncthreads();
+    sort_rods(o.rowP, o.rowQ, nr, reinterpret_cast<unsigned*>(o.U), reinterpret_cast<int*>(o.U) + nr, o.perm);
+}
+
+template <typename T>
+__device__ __forceinline__ int slot_gid(const Own1<T>& o, int t)
+{
+    return t < o.nc ? o.c0 + t : o.gid[t - o.nc];
+}
+
+// Rod phase over the block's rods, every entry from shared memory (modes
+// as for phase_a: A_STEP forms delta_{k+1} with alpha and leaves dU in
+// shared memory; A_PG returns this thread's share of pi.A.pi; A_REF leaves
+// Uref = M D gamma_ref (compensated in float32) in shared memory and in
+// the global Uref).
+template <typename T, int MODE>
+__device__ __forceinline__ T rod_pass1(const SolveArgs<T>& a, const Own1<T>& o, T alpha)
+{
+    constexpr bool COMP = MODE == A_REF && sizeof(T) == 4;
+    const bool has_comp = a.comp != nullptr;
+    const size_t mp = a.mp, np = a.np, nt = o.nt;
+    T fmf = T(0);
+#pragma unroll 1
+    for (int tt = threadIdx.x; tt < o.r1 - o.r0; tt += blockDim.x) {
+        const int li = (int)o.perm[tt], i = o.r0 + li;
+        Acc<T, COMP> Fa[6];
+#pragma unroll
+        for (int w = 0; w < 6; ++w) Fa[w].init(T(0));
+        {   // owned constraints: slots [rowP[li] - c0, rowP[li + 1] - c0)
+            const int e = o.rowP[li + 1] - o.c0;
+#pragma unroll 1
+            for (int t = o.rowP[li] - o.c0; t < e; ++t) {
+                const T dv = o.ds[t], gv = o.grs[t], gr = o.gam[t];
+                T rv[6];
+#pragma unroll
+                for (int w = 0; w < 6; ++w) rv[w] = o.rec[w * nt + t];
+                const bool bil = has_comp && (o.loc[t] & kBil);
+                const T v = a_value<MODE, T>(dv, gv, gr, alpha, bil);
+                if (MODE == A_PG && bil) fmf += __ldg(&a.comp[o.c0 + t]) * v * v;   // the spring's compliance term
+#pragma unroll
+                for (int w = 0; w < 6; ++w) Fa[w].add_prod(v, rv[w]);
+                if (COMP) {   // gamma_lo (held in grs during a reference pass) and the records' low parts
+                    const int c = o.c0 + t;
+                    const T gl = gv;
+                    T rl[6];
+                    lo_side(a.lop, a.rec_lo, mp, c, 3, rl);
+#pragma unroll
+                    for (int w = 0; w < 6; ++w) Fa[w].add_lo(fma(v, rl[w], gl * rv[w]));
+                }
+            }
+        }
+        {   // constraints owned by other rods (owned or ghost slots)
+            const int e = o.rowQ[li + 1] - o.q0;
+#pragma unroll 1
+            for (int k = o.rowQ[li] - o.q0; k < e; ++k) {
+                const unsigned qs = o.qslot[k];
+                const int t = (int)(qs & kLocal);
+                const T dv = o.ds[t], gv = o.grs[t], gr = o.gam[t];
+                T qv[6];
+#pragma unroll
+                for (int w = 0; w < 3; ++w) {
+                    qv[w] = o.rec[w * nt + t];
+                    qv[3 + w] = o.rec[(6 + w) * nt + t];
+                }
+                const T v = a_value<MODE, T>(dv, gv, gr, alpha, has_comp && (qs & kBil));
+#pragma unroll
+                for (int w = 0; w < 6; ++w) Fa[w].add_prod(-v, qv[w]);
+                if (COMP) {
+                    const int c = slot_gid(o, t);
+                    const T gl = gv;
+                    T ql[6];
+                    lo_side(a.loq, a.rec_lo, mp, c, 6, ql);
+#pragma unroll
+                    for (int w = 0; w < 6; ++w) Fa[w].add_lo(-fma(v, ql[w], gl * qv[w]));
+                }
+            }
+        }
+        T F[6];
+#pragma unroll
+        for (int w = 0; w < 6; ++w) F[w] = Fa[w].value();
+        const T p0 = o.ax[li], p1 = o.ax[o.cap_r + li], p2 = o.ax[2 * o.cap_r + li];
+        T ip = a.inv_perp, ipa = a.inv_par, ir = a.inv_rot, is = a.inv_spin;
+        if (a.mobr) {
+            ip = __ldg(&a.mobr[i]); ipa = __ldg(&a.mobr[np + i]);
+            ir = __ldg(&a.mobr[2 * np + i]); is = __ldg(&a.mobr[3 * np + i]);
+        }
+        const T p[3] = {p0, p1, p2};
+        T Uv[6];
+        half_mobility(p, F, ip, ipa, Uv);
+        half_mobility(p, F + 3, ir, is, Uv + 3);
+        if (MODE == A_PG) {
+#pragma unroll
+            for (int w = 0; w < 6; ++w) fmf += F[w] * Uv[w];
+        } else {
+#pragma unroll
+            for (int w = 0; w < 6; ++w) o.U[w * o.cap_r + li] = Uv[w];
+            if (MODE == A_REF) st_u6(a.Uref, i, Uv);
+        }
+    }
+    return fmf;
+}
+
+// The block's dU (shared [6][cap_r]) into its contiguous range of the
+// global [n][6] buffer dst, consecutive threads writing consecutive pairs.
+template <typename T>
+__device__ __forceinline__ void copy_out1(T* dst, const Own1<T>& o)
+{
+    __syncthreads();
+    const int nr = o.r1 - o.r0;
+    typename V2<T>::t* g = reinterpret_cast<typename V2<T>::t*>(dst + 6 * (size_t)o.r0);
+    for (int k = threadIdx.x; k < 3 * nr; k += blockDim.x) {
+        const int r = k / 3, w = 2 * (k - 3 * r);
+        typename V2<T>::t v;
+        v.x = o.U[w * o.cap_r + r];
+        v.y = o.U[(w + 1) * o.cap_r + r];
+        g[k] = v;
+    }
+}
+
+// Uref = 0 for the block's rods: shared memory and its rows of the global
+// Uref (the velocity the step reports if gamma_0 already meets the tolerance).
+template <typename T>
+__device__ __forceinline__ void zero_uref1(const SolveArgs<T>& a, const Own1<T>& o)
+{
+    const int nr = o.r1 - o.r0;
+    for (int k = threadIdx.x; k < 6 * o.cap_r; k += blockDim.x) o.U[k] = T(0);
+    typename V2<T>::t z;
+    z.x = T(0);
+    z.y = T(0);
+    typename V2<T>::t* g = reinterpret_cast<typename V2<T>::t*>(a.Uref + 6 * (size_t)o.r0);
+    for (int k = threadIdx.x; k < 3 * nr; k += blockDim.x) g[k] = z;
+}
+
+// The two velocities of slot t, P side first: Ui of the owner, Uj of the
+// other end (0 for a wall).  Local rods from shared memory, others from the
+// global buffer Ug.
+template <typename T>
+__device__ __forceinline__ void slot_velocities(const Own1<T>& o, int t, const T* Ug, T Ui[6], T Uj[6])
+{
+    const int li = (int)(o.loc[t] & kLocal);
+    const int ro = o.oth[t];
+    T Ul[6], Uo[6];
+#pragma unroll
+    for (int w = 0; w < 6; ++w) Ul[w] = o.U[w * o.cap_r + li];
+    if (ro < 0) {
+#pragma unroll
+        for (int w = 0; w < 6; ++w) Uo[w] = T(0);
+    } else if (ro >= o.r0 && ro < o.r1) {
+#pragma unroll
+        for (int w = 0; w < 6; ++w) Uo[w] = o.U[w * o.cap_r + (ro - o.r0)];
+    } else {
+        ld_u6(Ug, ro, Uo);
+    }
+    const bool own = t < o.nc;
+#pragma unroll
+    for (int w = 0; w < 6; ++w) {
+        Ui[w] = own ? Ul[w] : Uo[w];
+        Uj[w] = own ? Uo[w] : Ul[w];
+    }
+}
+
+// Constraint phase of a step over every slot: delta_k from
+// (delta_{k-1}, g_{k-1}, alpha_{k-1}) exactly as the rod phase formed it,
+// g_k = gref + D^T dU_k (+ the spring's compliance term), and for owned
+// slots acc = (s.s, s.y, y.y, max |pi|).
+template <typename T>
+__device__ __forceinline__ void con_pass_step1(const SolveArgs<T>& a, const Own1<T>& o, T alpha, const T* Ug, T acc[4])
+{
+    const bool has_comp = a.comp != nullptr;
+    const size_t nt = o.nt;
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
+        T Ui[6], Uj[6], r[9];
+        slot_velocities(o, t, Ug, Ui, Uj);
+#pragma unroll
+        for (int w = 0; w < 9; ++w) r[w] = o.rec[w * nt + t];
+        const T dold = o.ds[t], gro = o.grs[t], gam = o.gam[t];
+        const int c = slot_gid(o, t);
+        const T cmp = has_comp ? __ldg(&a.comp[c]) : T(-1);
+        const bool bil = cmp >= T(0);
+        const T dm = a_value<A_STEP, T>(dold, gro, gam, alpha, bil);
+        Acc<T, false> du;
+        du.init(o.gref[t]);
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            du.add_prod(r[u], Ui[u]);
+            du.add_prod(-r[u], Uj[u]);
+            du.add_prod(r[3 + u], Ui[3 + u]);
+            du.add_prod(-r[6 + u], Uj[3 + u]);
+        }
+        if (bil) du.add_prod(cmp, dm);
+        const T gr = du.value();
+        o.ds[t] = dm;
+        o.grs[t] = gr;
+        if (t < o.nc) {
+            const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
+            const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
+            acc[3] = api > acc[3] ? api : acc[3];
+            const T sv = dm - dold, yv = gr - gro;
+            acc[0] += sv * sv;
+            acc[1] += sv * yv;
+            acc[2] += yv * yv;
+        }
+    }
+}
+
+// Constraint phase of a refresh over every slot: gref = q + D^T Uref from
+// the split records and q with compensated sums (float32), g = gref, and
+// for owned slots acc = (pi.pi, 0, 0, max |pi|) at gamma_ref.  ZERO: Uref
+// is 0 (gamma_ref = 0), so no velocity is read and the records' products
+// (all zero) are left out of the sums.
+template <typename T, bool ZERO = false>
+__device__ __forceinline__ void con_pass_ref1(const SolveArgs<T>& a, const Own1<T>& o, T acc[4])
+{
+    constexpr bool COMP = sizeof(T) == 4;
+    const bool has_comp = a.comp != nullptr;
+    const size_t nt = o.nt, mp = a.mp;
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
+        T Ui[6], Uj[6], r[9];
+        if (!ZERO) {
+            slot_velocities(o, t, a.Uref, Ui, Uj);
+#pragma unroll
+            for (int w = 0; w < 9; ++w) r[w] = o.rec[w * nt + t];
+        }
+        const int c = slot_gid(o, t);
+        const T gam = o.gam[t];
+        Acc<T, COMP> du;
+        du.init(__ldg(&a.q[c]));
+        if (!ZERO) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+                du.add_prod(r[u], Ui[u]);
+                du.add_prod(-r[u], Uj[u]);
+                du.add_prod(r[3 + u], Ui[3 + u]);
+                du.add_prod(-r[6 + u], Uj[3 + u]);
+            }
+        }
+        const T cmp = has_comp ? __ldg(&a.comp[c]) : T(-1);
+        const bool bil = cmp >= T(0);
+        if (bil) {
+            du.add_prod(cmp, gam);
+            du.add_lo(cmp * o.grs[t]);   // gamma_lo, before g takes its place below
+        }
+        if (COMP) {
+            T tl = __ldg(&a.q_lo[c]);
+            if (!ZERO) {
+                T lp[6], lq[6];   // (e, y_P x e) and (e, y_Q x e) low parts
+                lo_side(a.lop, a.rec_lo, mp, c, 3, lp);
+                lo_side(a.loq, a.rec_lo, mp, c, 6, lq);
+#pragma unroll
+                for (int u = 0; u < 3; ++u)
+                    tl += fma(-lq[3 + u], Uj[3 + u], fma(lp[u], Ui[u] - Uj[u], lp[3 + u] * Ui[3 + u]));
+            }
+            du.add_lo(tl);
+        }
+        const T gr = du.value();
+        o.gref[t] = gr;
+        o.grs[t] = gr;
+        if (t < o.nc) {
+            const T dm = o.ds[t];   // 0 after the fold
+            const T pi = (bil || dm > -gam) ? gr : (gr < T(0) ? gr : T(0));
+            const T api = (pi < T(0) ? -pi : pi) * __ldg(&a.isc[c]);
+            acc[3] = api > acc[3] ? api : acc[3];
+            acc[0] += pi * pi;
+        }
+    }
+}
+
+// Refresh, first half: every slot folds delta into (gamma_ref, gamma_lo)
+// as fold_delta does, from the previous reference's gamma_lo in gprev;
+// ghosts repeat their owner's arithmetic on the same inputs, so both hold
+// the same reference without waiting for each other.  gamma_ref goes to
+// gam, gamma_lo to grs (the reference passes' low part, until the constraint
+// pass replaces it by g), and owned slots publish (gamma_ref, gamma_lo) in
+// gnew, the other state buffer (ghosts are still reading gprev).
+template <typename T>
+__device__ __forceinline__ void fold1(const SolveArgs<T>& a, const Own1<T>& o, const T* gprev, T* gnew)
+{
+    const bool has_comp = a.comp != nullptr;
+#pragma unroll 1
+    for (int t = threadIdx.x; t < o.nt; t += blockDim.x) {
+        const int c = slot_gid(o, t);
+        const T d = o.ds[t], gr = o.gam[t], gl = gl_of_state(gprev, c);
+        const bool bil = has_comp && (o.loc[t] & kBil);
+        T hi = T(0), lo = T(0);
+        if (bil || d > -gr) {
+            T s, e;
+            two_sum(gr, d, s, e);
+            const T l = gl + e;
+            hi = s + l;
+            lo = l - (hi - s);
+            if (!bil && (hi < T(0) || (hi == T(0) && lo < T(0)))) { hi = T(0); lo = T(0); }
+        }
+        o.gam[t] = hi;
+        o.grs[t] = lo;
+        o.ds[t] = T(0);
+        if (t < o.nc) st_ref(gnew, c, hi, lo);
+    }
+}
+
+// cp.async of the last barrier's block sums ([4][nbp] of buffer src) into
+// shared memory; the threads that issue it wait for it in tot_wait.
+template <typename T>
+__device__ __forceinline__ void tot_fetch(const Own1<T>& o, const T* src)
+{
+    const int chunks = (int)(4 * (size_t)o.nbp * sizeof(T) / 16);
+    if ((int)threadIdx.x < chunks) {
+        for (int q = threadIdx.x; q < chunks; q += blockDim.x) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(reinterpret_cast<unsigned char*>(o.tot) + 16 * (size_t)q);
+            const unsigned char* s = reinterpret_cast<const unsigned char*>(src) + 16 * (size_t)q;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(s) : "memory");
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+}
+__device__ __forceinline__ void tot_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Warp w's share of the block sums: each warp's (sum, sum, sum, max) into red[w].
+template <typename T>
+__device__ __forceinline__ void warp_partial(T v[4], T (*red)[4])
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) v[u] += __shfl_down_sync(0xffffffffu, v[u], o);
+        const T mx = __shfl_down_sync(0xffffffffu, v[3], o);
+        v[3] = mx > v[3] ? mx : v[3];
+    }
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) red[threadIdx.x >> 5][u] = v[u];
+    }
+}
+
+// Warp 0 after a block barrier: the block's sums over red, lane 0 stores
+// them in dst ([4][stride]).
+template <typename T>
+__device__ __forceinline__ void block_store(T (*red)[4], T* dst, int stride)
+{
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    T w[4] = {T(0), T(0), T(0), T(0)};
+    if (lane < nw) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = red[lane][u];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) w[u] += __shfl_down_sync(0xffffffffu, w[u], o);
+        const T mx = __shfl_down_sync(0xffffffffu, w[3], o);
+        w[3] = mx > w[3] ? mx : w[3];
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dst[u * stride + blockIdx.x] = w[u];
+    }
+}
+
+// One warp: the grid total of row u of the fetched block sums (sums for
+// u < 3, the maximum for u = 3), in a fixed order, so every block gets the
+// same numbers; every lane returns it.
+template <typename T>
+__device__ __forceinline__ T row_total(const Own1<T>& o, int nb, int u)
+{
+    const int lane = threadIdx.x & 31;
+    const T* row = o.tot + (size_t)u * o.nbp;
+    T w = T(0);
+    for (int b = lane; b < nb; b += 32) {
+        const T x = row[b];
+        w = u == 3 ? (x > w ? x : w) : w + x;
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const T y = __shfl_xor_sync(0xffffffffu, w, s);
+        w = u == 3 ? (y > w ? y : w) : w + y;
+    }
+    return w;
+}
+
+// The four totals, one warp each: warps 1-4 store them in shared memory and
+// meet on a named barrier (warp 0 meanwhile stores the block's own sums).
+template <typename T>
+__device__ __forceinline__ void warps_totals(const Own1<T>& o, int nb, T* tot)
+{
+    const int u = (int)(threadIdx.x >> 5) - 1;
+    const T w = row_total(o, nb, u);
+    if ((threadIdx.x & 31) == 0) tot[u] = w;
+    asm volatile("bar.sync 1, 128;\n" ::: "memory");
+}
+
+// Loop states: what the last constraint phase was (its sums are what the
+// last barrier published), and the decision taken for the next rod phase.
+
+template <typename T>
+__global__ void __launch_bounds__(1024, 1) k_bbpgd1_meet(SolveArgs<T> a)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ Shared1<T> sh;
+    if (a.fault == 1 && blockIdx.x == 0) return;   // test hook: this block never arrives
+    Own1<T> o;
+    o.r0 = a.bstart[blockIdx.x];
+    o.r1 = a.bstart[blockIdx.x + 1];
+    o.c0 = a.rowP[o.r0];
+    o.c1 = a.rowP[o.r1];
+    o.q0 = a.rowQ[o.r0];
+    o.q1 = a.rowQ[o.r1];
+    o.nc = o.c1 - o.c0;
+    o.cap_r = o.r1 - o.r0;
+    const int nb = (int)gridDim.x;
+    o.nbp = (nb + 3) & ~3;
+    stage_in1(a, o, dyn, sh);
+    T* const dU2 = reinterpret_cast<T*>(a.xch);   // the second velocity buffer [n][6]
+    T* part = reinterpret_cast<T*>(a.partials);   // [2][4][nbp]
+    const size_t pstride = 4 * (size_t)o.nbp;
+    unsigned epoch = 0;
+    int* s_ok = &sh.ng;   // the barrier's broadcast word (ng is not needed after staging)
+    auto barrier = [&]() { return grid_barrier(a.bar, (unsigned)nb * ++epoch, a.flags, a.wait_cycles, s_ok); };
+    const int warp = threadIdx.x >> 5;
+    // step state, kept by thread 32 (warp 1, lane 0)
+    T alpha0 = T(1), pimax = T(0);
+    int k = 0, since = 0, hist = 0;
+    bool ok = true;
+
+    // initial reference at gamma_0 and the line step alpha_0 = pi.pi / pi.A.pi;
+    // from gamma_0 = 0, Uref = M D gamma_0 = 0 needs no rod pass and no
+    // other block's velocities
+    if (a.zero_start) {
+        zero_uref1(a, o);
+        __syncthreads();
+    } else {
+        rod_pass1<T, A_REF>(a, o, T(0));
+        ok = barrier();
+    }
+    int pw = 0;   // block-sum buffer the next barrier publishes
+    if (ok) {
+        T v[4] = {T(0), T(0), T(0), T(0)};
+        if (a.zero_start) con_pass_ref1<T, true>(a, o, v);
+        else con_pass_ref1(a, o, v);
+        __syncthreads();   // gref and g of every slot before the line step reads them
+        v[1] = rod_pass1<T, A_PG>(a, o, T(0));
+        warp_partial(v, sh.red);
+        __syncthreads();
+        if (warp == 0) block_store(sh.red, part + pw * pstride, o.nbp);
+        ok = barrier();
+    }
+    if (ok) {
+        tot_fetch(o, part + pw * pstride);
+        tot_wait();
+        __syncthreads();
+        if (warp >= 1 && warp <= 4) {
+            warps_totals(o, nb, sh.tot);
+            const T* tot = sh.tot;
+            if (threadIdx.x == 32) {
+                pimax = tot[3];
+                const double pap = (double)tot[1];
+                double al = (double)tot[0] / pap;
+                if (!(pap > 0.0) || !isfinite(al) || !(al > 0.0) || !isfinite((T)al)) al = 1.0;
+                alpha0 = (T)al;
+                sh.alpha = alpha0;
+                sh.kind = (!above_tol(a, pimax) || a.max_iter <= 0) ? K_STOP1 : K_STEP1;
+            }
+        }
+        __syncthreads();
+        pw ^= 1;
+    }
+    int cprev = C_NONE1;      // the constraint phase whose sums the last barrier published
+    bool rstep = false;       // the last rod phase formed a step (its delta is still to be stored)
+    T alpha_prev = T(0);
+    int db = 0;               // dU buffer the next step's rod phase writes
+    int nref = 0;             // refreshes taken: the reference lives in state buffer nref & 1
+    while (ok && sh.kind != K_STOP1) {
+        const int pr = pw ^ 1;   // buffer the last barrier published
+        if (cprev != C_NONE1) tot_fetch(o, part + pr * pstride);
+        T v[4] = {T(0), T(0), T(0), T(0)};
+        if (rstep) con_pass_step1(a, o, alpha_prev, db ? a.U : dU2, v);
+        const int ccur = rstep ? C_STEP1 : C_NONE1;
+        warp_partial(v, sh.red);
+        tot_wait();
+        __syncthreads();
+        if (warp == 0) {
+            block_store(sh.red, part + pw * pstride, o.nbp);
+        } else if (warp <= 4) {
+            if (cprev != C_NONE1) warps_totals(o, nb, sh.tot);
+            const T* tot = sh.tot;
+            if (threadIdx.x == 32) {
+                if (rstep) ++k;
+                int kind = K_STEP1;
+                T an = sh.alpha;
+                if (cprev == C_STEP1) {
+                    // sums of (s_{k-2}, y_{k-2}) and max |pi| at the iterate before the slots'
+                    pimax = tot[3];
+                    ++since;
+                    const bool below = !above_tol(a, pimax);
+                    if ((below && since >= 2) || (a.refresh > 0 && since >= a.refresh) || k >= a.max_iter) {
+                        kind = K_REF1;
+                    } else {
+                        const T ss = tot[0], sy = tot[1], yy = tot[2];
+                        an = (hist & 1) == 0 ? ss / sy : sy / yy;
+                        if (!(sy > T(0)) || !isfinite(an) || !(an > T(0))) an = alpha0;
+                        ++hist;
+                    }
+                } else if (cprev == C_REF1) {
+                    // the fresh reference's exact residual: the slots' step from it is dropped on a stop
+                    pimax = tot[3];
+                    since = 0;
+                    if (!above_tol(a, pimax) || k - 1 >= a.max_iter) {
+                        kind = K_STOP1;
+                        --k;
+                    }
+                } else if (k >= a.max_iter) {
+                    kind = K_REF1;   // the cap reached before any step's sums came back
+                }
+                sh.alpha = an;
+                sh.kind = kind;
+            }
+        }
+        __syncthreads();
+        const int kind = sh.kind;
+        if (kind == K_STOP1) break;
+        int cpub = ccur;
+        if (kind == K_REF1) {
+            fold1(a, o, nref & 1 ? a.gg1 : a.gg0, nref & 1 ? a.gg0 : a.gg1);
+            ++nref;
+            __syncthreads();
+            rod_pass1<T, A_REF>(a, o, T(0));
+            if (!(ok = barrier())) break;
+            T w[4] = {T(0), T(0), T(0), T(0)};
+            con_pass_ref1(a, o, w);
+            warp_partial(w, sh.red);
+            __syncthreads();
+            if (warp == 0) block_store(sh.red, part + pw * pstride, o.nbp);
+            cpub = C_REF1;
+        }
+        const T al = sh.alpha;
+        rod_pass1<T, A_STEP>(a, o, al);
+        copy_out1(db ? dU2 : a.U, o);
+        alpha_prev = al;
+        rstep = true;
+        db ^= 1;
+        if (!(ok = barrier())) break;
+        pw ^= 1;
+        cprev = cpub;
+    }
+    if (!ok) return;
+    // every solve ends on a fresh reference: gamma = gamma_ref + gamma_lo
+    // (state buffer nref & 1) and delta = 0, so dU = 0
+    T* gfin = nref & 1 ? a.gg1 : a.gg0;
+    for (int t = threadIdx.x; t < o.nc; t += blockDim.x) st_dg(gfin, o.c0 + t, T(0), o.gref[t]);
+    {
+        typename V2<T>::t z;
+        z.x = T(0);
+        z.y = T(0);
+        typename V2<T>::t* g = reinterpret_cast<typename V2<T>::t*>(a.U + 6 * (size_t)o.r0);
+        for (int q = threadIdx.x; q < 3 * (o.r1 - o.r0); q += blockDim.x) g[q] = z;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 32) {
+        a.out[1] = (double)alpha0;
+        a.flags[F_FINAL] = nref & 1;
+        a.flags[F_ITERS] = k;
+        a.out[0] = a.hD * (double)pimax;
+    }
+}
+
+}  // namespace meet
+
 // The work-balanced split and what its shares need, one thread block per solver block b
 // in one launch (three before): the share's two boundaries (bstart; a warp
 // each), the two-barrier kernel's largest shared-memory share and rod count
@@ -2761,10 +3465,45 @@ static int threads1(const aLENS_ctx* ctx)
 
 static_assert(sizeof(Shared1<double>) <= sizeof(Shared<double>) + 768 && sizeof(Shared1<float>) <= sizeof(Shared<float>) + 768,
               "the one-barrier kernel's static shared memory and the shares' budget exceed a block's limit");
-template <typename T>
-static const void* kernel1(const aLENS_ctx* ctx)
+// The one-barrier kernel of a launch: for caller order, for the default shape
+// (80 registers a thread), for the others; several blocks on an SM share its registers.
+enum { V_MEET = 0, V_WIDE = 1, V_ANY = 2 };
+static int variant1(const aLENS_ctx* ctx, int n)
 {
-    return threads1(ctx) <= kThreads1 ? (const void*)k_bbpgd1<T, kThreads1> : (const void*)k_bbpgd1<T, 1024>;
+    if (ctx->caller_order && n > kMeetRods) return V_MEET;
+    return threads1(ctx) <= kThreads1 && ctx->solve_bps <= 1 ? V_WIDE : V_ANY;
+}
+template <typename T>
+static const void* kernel1(int variant)
+{
+    return variant == V_MEET   ? (const void*)meet::k_bbpgd1_meet<T>
+           : variant == V_WIDE ? (const void*)k_bbpgd1<T, kThreads1>
+                               : (const void*)k_bbpgd1<T, 1024>;
+}
+// Its threads, and whether bps blocks of it fit an SM with `budget` bytes of
+// dynamic shared memory each (occupancy only falls as shared memory grows: one
+// answer per shape; the limit on dynamic shared memory is set once per kernel).
+template <typename T>
+static cudaError_t ready1(aLENS_ctx* ctx, int variant, size_t budget, int& threads, bool& fits)
+{
+    const int ti = sizeof(T) == 4 ? 0 : 1, bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
+    const void* fn = kernel1<T>(variant);
+    threads = variant == V_MEET ? ctx->solve_threads : threads1(ctx);
+    cudaError_t e;
+    if (!(ctx->attr1_set[ti] & 1 << variant)) {
+        const long long most = (long long)ctx->smem_optin - (long long)sizeof(Shared1<T>) - 256;
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most)) != cudaSuccess) return e;
+        ctx->attr1_set[ti] |= 1 << variant;
+    }
+    const int key = (variant * 2048 + ctx->solve_threads) * 64 + bps;
+    if (ctx->occ1_key[ti] != key) {
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, budget)) != cudaSuccess) return e;
+        ctx->occ1_ok[ti] = per_sm >= bps;
+        ctx->occ1_key[ti] = key;
+    }
+    fits = ctx->occ1_ok[ti] != 0;
+    return cudaSuccess;
 }
 
 template <typename T>
@@ -2802,35 +3541,19 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     const long long budget = (long long)optin / bps - (long long)sizeof(Shared<T>) - 1024;
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
         // one grid barrier per iteration: every block's share and its ghosts fit
-        const void* fn1 = kernel1<T>(ctx);
-        const int ti = sizeof(T) == 4 ? 0 : 1;
-        const long long budget1 = (long long)optin - (long long)sizeof(Shared1<T>) - 256;   // the most a block may ask for
-        if (!ctx->attr1_set[ti]) {
-            // the limit for the largest budget once; a launch asks for its own need
-            if ((e = cudaFuncSetAttribute(fn1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget1)) !=
-                cudaSuccess)
-                return e;
-            ctx->attr1_set[ti] = 1;
-        }
-        // occupancy only falls as shared memory grows: checked once per shape at the full budget
-        const int key = threads * 64 + bps;
-        if (ctx->occ1_key[ti] != key) {
-            int per_sm1 = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads1(ctx), (size_t)budget)) !=
-                cudaSuccess)
-                return e;
-            ctx->occ1_ok[ti] = per_sm1 >= bps;
-            ctx->occ1_key[ti] = key;
-        }
-        if (ctx->occ1_ok[ti] && (long long)bps * ctx->num_sms >= blocks) {
+        const int variant = variant1(ctx, n);
+        int threads = 0;
+        bool fits = false;
+        if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
+        if (fits && (long long)bps * ctx->num_sms >= blocks) {
             // the share proper, with room for ds and gs (2 values for 13) and for
             // a halo rod (6 values) per slot
             const long long room = (long long)need1 + (long long)need1 * 8 / 13;
-            a.dyn_bytes = (size_t)(room < budget ? room : budget);
+            a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : room < budget ? room : budget);
             void* args1[] = {&a};
             ++ctx->launches;
             ctx->last_solver = 1;
-            return cudaLaunchCooperativeKernel(fn1, dim3((unsigned)blocks), dim3(threads1(ctx)), args1, a.dyn_bytes,
+            return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, a.dyn_bytes,
                                                ctx->stream);
         }
     }
@@ -2990,23 +3713,9 @@ template <typename T>
 static cudaError_t graph1_check(aLENS_ctx* ctx, bool& ok)
 {
     ok = false;
-    const int threads = ctx->solve_threads, bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
-    if (ctx->solve_barriers != 1 || threads < 256) return cudaSuccess;
-    const void* fn1 = kernel1<T>(ctx);
-    const int ti = sizeof(T) == 4 ? 0 : 1;
-    const long long budget1 = (long long)ctx->smem_optin - (long long)sizeof(Shared1<T>) - 256;
-    cudaError_t e;
-    if (!ctx->attr1_set[ti]) {
-        if ((e = cudaFuncSetAttribute(fn1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget1)) != cudaSuccess)
-            return e;
-        ctx->attr1_set[ti] = 1;
-    }
-    int per_sm1 = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, fn1, threads1(ctx),
-                                                           (size_t)graph1_budget<T>(ctx))) != cudaSuccess)
-        return e;
-    ok = per_sm1 >= bps;
-    return cudaSuccess;
+    if (ctx->solve_barriers != 1 || ctx->solve_threads < 256) return cudaSuccess;
+    int threads = 0;
+    return ready1<T>(ctx, variant1(ctx, 0), (size_t)graph1_budget<T>(ctx), threads, ok);
 }
 
 template <typename T>
@@ -3033,8 +3742,8 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
-    return cudaLaunchCooperativeKernel(kernel1<T>(ctx), dim3((unsigned)blocks), dim3(threads1(ctx)),
-                                       args1, (size_t)budget, ctx->stream);
+    return cudaLaunchCooperativeKernel(kernel1<T>(variant1(ctx, 0)), dim3((unsigned)blocks), dim3(threads1(ctx)), args1,
+                                       (size_t)budget, ctx->stream);
 }
 
 cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)
