@@ -13,9 +13,10 @@
 //     s.s / s.y and s.y / y.y in turn (alternating BB1/BB2): the
 //     Barzilai-Borwein step taken one iteration late, a gradient method with
 //     retards (Friedlander, Martinez, Molina & Raydan, SIAM J. Numer. Anal.
-//     36, 1999), which lets the one-barrier solver below form the step
-//     length from sums that arrive with the next barrier; every solver kernel
-//     uses it, so all of them run one method;
+//     36, 1999), which lets the one-barrier solver below (at most one grid
+//     barrier an iteration) form the step length from sums that arrive while
+//     another phase runs; every solver kernel uses it, so all of them run
+//     one method;
 //   alpha_0 = pi.pi / pi.A.pi for the projected gradient pi at gamma_0, for
 //   the first two steps and whenever s.y <= 0 or the step is not finite.
 // Stop when (h/D) max |pi_c| <= tol (pi the projected gradient) or after
@@ -65,6 +66,7 @@
 
 #include <cmath>
 #include <limits>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -547,6 +549,87 @@ __device__ __forceinline__ T phase_a(const SolveArgs<T>& a, const Own<T>& o, int
         }
     }
     return fmf;
+}
+
+// Velocity M F of one rod, three components: a n F + p (p.F)(b - a), the
+// translational half (a = 1/zeta_perp, b = 1/zeta_par) or the rotational
+// one.  The products' fusing is written out, so that every kernel rounds alike.
+template <typename T>
+__device__ __forceinline__ void half_mobility(const T p[3], const T F[3], T ia, T ib, T U[3])
+{
+    const T pf = fma(p[2], F[2], fma(p[0], F[0], p[1] * F[1]));
+    const T cf = pf * (ib - ia);
+#pragma unroll
+    for (int w = 0; w < 3; ++w) U[w] = fma(p[w], cf, F[w] * ia);
+}
+
+// Rod phase of a float32 step of the batched solver: one thread per rod over
+// its entries, owned then other-side, in one loop; the next entry's state and
+// row and the id of the one after are loaded while the current one is summed.
+// A cluster's blocks have too few rods to hide the loads of one entry behind
+// other warps' (solve, 256 systems 21.5 -> 20.8 ms, 16 small ones 2.52 -> 2.38;
+// the single-system solver, whose loads L2 and HBM bound, is 6 to 9 % slower this
+// way on the 4e5-rod pack and keeps phase_a's two loops).
+__device__ __forceinline__ void rod_step_g(const SolveArgs<float>& a, const Own<float>& o, int cur, float alpha)
+{
+    const float4* const gc = reinterpret_cast<const float4*>(cur ? a.gg1 : a.gg0);
+    const size_t np = a.np;
+    const bool has_comp = a.comp != nullptr;
+#pragma unroll 1
+    for (int i = o.r0 + threadIdx.x; i < o.r1; i += blockDim.x) {
+        const int b = a.rowP[i], no = a.rowP[i + 1] - b, k0 = a.rowQ[i] - no, ne = no + a.rowQ[i + 1] - a.rowQ[i];
+        float F[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        auto id = [&](int e) { return e < no ? b + e : e < ne ? __ldg(&a.qlist[k0 + e]) : 0; };
+        auto row = [&](int e, int c) {
+            return reinterpret_cast<const float4*>(e < no ? a.pe : a.qe) + 2 * (size_t)(e < no ? c : k0 + e);
+        };
+        int c = id(0), c1 = id(1);
+        float4 st = make_float4(0.0f, 0.0f, 0.0f, 0.0f), ra = st;
+        float2 rb = make_float2(0.0f, 0.0f);
+        if (ne > 0) {
+            st = gc[c];
+            const float4* const p = row(0, c);
+            ra = __ldg(p);
+            rb = __ldg(reinterpret_cast<const float2*>(p + 1));
+        }
+#pragma unroll 1
+        for (int e = 0; e < ne; ++e) {
+            float4 st1 = st, ra1 = ra;
+            float2 rb1 = rb;
+            if (e + 1 < ne) {
+                st1 = gc[c1];
+                const float4* const p = row(e + 1, c1);
+                ra1 = __ldg(p);
+                rb1 = __ldg(reinterpret_cast<const float2*>(p + 1));
+            }
+            const int c2 = id(e + 2);
+            bool bil = false;
+            if (has_comp) bil = __ldg(&a.comp[c]) >= 0.0f;
+            const float v = a_value<A_STEP, float>(st.x, st.y, st.z, alpha, bil);
+            const float w = e < no ? v : -v;
+            F[0] = fma(w, ra.x, F[0]);
+            F[1] = fma(w, ra.y, F[1]);
+            F[2] = fma(w, ra.z, F[2]);
+            F[3] = fma(w, ra.w, F[3]);
+            F[4] = fma(w, rb.x, F[4]);
+            F[5] = fma(w, rb.y, F[5]);
+            st = st1;
+            ra = ra1;
+            rb = rb1;
+            c = c1;
+            c1 = c2;
+        }
+        const float p[3] = {a.ax[i], a.ax[np + i], a.ax[2 * np + i]};
+        float ip = a.inv_perp, ipa = a.inv_par, ir = a.inv_rot, is = a.inv_spin;
+        if (a.mobr) {
+            ip = __ldg(&a.mobr[i]); ipa = __ldg(&a.mobr[np + i]);
+            ir = __ldg(&a.mobr[2 * np + i]); is = __ldg(&a.mobr[3 * np + i]);
+        }
+        float U[6];
+        half_mobility(p, F, ip, ipa, U);
+        half_mobility(p, F + 3, ir, is, U + 3);
+        st_u6(a.U, i, U);
+    }
 }
 
 // A staged step's dU for the other blocks: the block's rods [r0, r1) are
@@ -1091,7 +1174,11 @@ __device__ __forceinline__ void solve_loop(const SolveArgs<T>& a, const Own<T>& 
         const int nx = cur ^ 1;
         v[0] = v[1] = v[2] = v[3] = T(0);
         if (kind == P_STEP) {
-            phase_a<T, A_STEP, ST>(a, o, cur, sh.alpha);
+            if constexpr (!ST && sizeof(T) == 4 && std::is_same<SY, BatchSync<T>>::value) {
+                rod_step_g(a, o, cur, sh.alpha);
+            } else {
+                phase_a<T, A_STEP, ST>(a, o, cur, sh.alpha);
+            }
             if (ST) copy_out_du(a, o);
             if (!sy.barrier(sh)) return;
             phase_b<T, B_STEP, ST>(a, o, cur, nx, sh.alpha, v);
@@ -1731,18 +1818,6 @@ __device__ __forceinline__ void lo_side(const T* rows, const T* rec_lo, size_t m
         out[w] = __ldg(&rec_lo[w * mp + c]);
         out[3 + w] = __ldg(&rec_lo[(arm0 + w) * mp + c]);
     }
-}
-
-// Velocity M F of one rod, three components: a n F + p (p.F)(b - a), the
-// translational half (a = 1/zeta_perp, b = 1/zeta_par) or the rotational
-// one.  The products' fusing is written out, so that every kernel rounds alike.
-template <typename T>
-__device__ __forceinline__ void half_mobility(const T p[3], const T F[3], T ia, T ib, T U[3])
-{
-    const T pf = fma(p[2], F[2], fma(p[0], F[0], p[1] * F[1]));
-    const T cf = pf * (ib - ia);
-#pragma unroll
-    for (int w = 0; w < 3; ++w) U[w] = fma(p[w], cf, F[w] * ia);
 }
 
 // Rod pass of the reference (one thread per rod): A_REF leaves Uref = M D
