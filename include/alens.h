@@ -111,8 +111,8 @@ typedef struct {
     float ms_solve;     /* device time of the BBPGD kernel alone */
     float ms_update;    /* device time of the update */
     int32_t launches;   /* kernels the call launched */
-    int32_t solver;     /* solver kernel of the call: 0 none, 1 one grid barrier per
-                           iteration, 2 two barriers with shared-memory shares,
+    int32_t solver;     /* solver kernel of the call: 0 none, 1 at most one grid barrier
+                           per iteration, 2 two barriers with shared-memory shares,
                            3 two barriers from global memory, 4 per-system clusters */
 } aLENS_info;
 
