@@ -897,7 +897,7 @@ def run_ours(args):
         "data": "synthetic",
         "config": config,
         "bbpgd_iters": statistics.mean(it), "residual": res, "launch_shape": tuned,
-        "solver_kernel": {0: None, 1: "one grid barrier per iteration", 2: "two barriers, shared-memory shares",
+        "solver_kernel": {0: None, 1: "shared-memory shares, at most one grid barrier per iteration", 2: "two barriers, shared-memory shares",
                           3: "two barriers, global memory", 4: "per-system clusters"}.get(infos[-1].get("solver")),
         "phase_ms": {k: statistics.mean(i[k] for i in infos) for k in ("ms_build", "ms_assemble", "ms_solve",
                                                                          "ms_update", "ms_adjoint") if k in infos[0]},

@@ -3615,7 +3615,7 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     const int optin = ctx->smem_optin;
     const long long budget = (long long)optin / bps - (long long)sizeof(Shared<T>) - 1024;
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
-        // one grid barrier per iteration: every block's share and its ghosts fit
+        // at most one grid barrier per iteration: every block's share and its ghosts fit
         const int variant = variant1(ctx, n);
         int threads = 0;
         bool fits = false;
@@ -3641,8 +3641,9 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     a.sort_cap = (int)maxrods;
     const size_t smem = staged ? (size_t)need : (a.sort_ns ? (size_t)sort_bytes : 0);
     constexpr int kMaxT = sizeof(T) == 8 ? 768 : 1024;
-    const void* fn = threads <= kMaxT ? (staged ? (const void*)k_bbpgd<T, true, kMaxT> : (const void*)k_bbpgd<T, false, kMaxT>)
-                                      : (staged ? (const void*)k_bbpgd<T, true, 1024> : (const void*)k_bbpgd<T, false, 1024>);
+    // (several blocks on an SM share its registers: 64 a thread there as well)
+    const void* fn = threads <= kMaxT && bps <= 1 ? (staged ? (const void*)k_bbpgd<T, true, kMaxT> : (const void*)k_bbpgd<T, false, kMaxT>)
+                                                  : (staged ? (const void*)k_bbpgd<T, true, 1024> : (const void*)k_bbpgd<T, false, 1024>);
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     int per_sm = 0;

@@ -6,8 +6,8 @@ float64 at tol 1e-10, 2e-5 D mixed at tol 1e-6).  The sizes sit at the edges of 
 kernel's layout: one block and its neighbours (32 rods a block until every SM has
 one), the last share whose rods get eight lanes (96 rods a block at 768
 workers) and the first that get two, a rod count just past a warp, shapes
-with and without a warp for the block sums (768 and 256; 1024; two blocks an
-SM), walls (the zero velocity row) and springs (bilateral slots), and a
+with and without a warp for the block sums (768 and 256; 1024; two and four
+blocks an SM), walls (the zero velocity row) and springs (bilateral slots), and a
 solve_lcp in the caller's order (a halo of nearly every slot's other end).
 """
 import numpy as np
@@ -66,9 +66,10 @@ def test_sizes(n, precision):
     steps(system(n), precision, 768, 0)
 
 
-@pytest.mark.parametrize("threads,bps", [(256, 1), (992, 1), (1024, 1), (512, 2)])
-def test_launch_shapes(threads, bps):
-    steps(system(3000), A.MIXED, threads, bps)
+@pytest.mark.parametrize("precision", [A.FP64, A.MIXED])
+@pytest.mark.parametrize("threads,bps", [(256, 1), (992, 1), (1024, 1), (512, 2), (256, 4)])
+def test_launch_shapes(threads, bps, precision):
+    steps(system({1: 3000, 2: 10000, 4: 20000}[bps]), precision, threads, bps)   # (every SM full of blocks)
 
 
 @pytest.mark.parametrize("precision", [A.FP64, A.MIXED])
