@@ -3044,6 +3044,13 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd1_meet(SolveArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ Shared1<T> sh;
+    if (a.need1_dev) {   // recorded step: as in k_bbpgd1
+        const unsigned long long need = *a.need1_dev;
+        if (need == 0 || need > (unsigned long long)a.fit_cap) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) a.flags[F_SOLVE_ERR] = kSolveRedo;
+            return;
+        }
+    }
     if (a.fault == 1 && blockIdx.x == 0) return;   // test hook: this block never arrives
     Own1<T> o;
     o.r0 = a.bstart[blockIdx.x];
@@ -3540,12 +3547,15 @@ static int threads1(const aLENS_ctx* ctx)
 
 static_assert(sizeof(Shared1<double>) <= sizeof(Shared<double>) + 768 && sizeof(Shared1<float>) <= sizeof(Shared<float>) + 768,
               "the one-barrier kernel's static shared memory and the shares' budget exceed a block's limit");
-// The one-barrier kernel of a launch: for caller order, for the default shape
-// (80 registers a thread), for the others; several blocks on an SM share its registers.
+// The one-barrier kernel of a launch: with the barrier for large systems in
+// caller order or with 1024 workers (no room for a warp of the sums' own: 1e5
+// rods 10.8 us an iteration against 13.3), without it in the default shape (72
+// registers a thread) and in the others (several blocks on an SM share its
+// registers).
 enum { V_MEET = 0, V_WIDE = 1, V_ANY = 2 };
 static int variant1(const aLENS_ctx* ctx, int n)
 {
-    if (ctx->caller_order && n > kMeetRods) return V_MEET;
+    if ((ctx->caller_order || (ctx->solve_threads > 992 && ctx->solve_bps <= 1)) && n > kMeetRods) return V_MEET;
     return threads1(ctx) <= kThreads1 && ctx->solve_bps <= 1 ? V_WIDE : V_ANY;
 }
 template <typename T>
@@ -3818,8 +3828,13 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
-    return cudaLaunchCooperativeKernel(kernel1<T>(variant1(ctx, 0)), dim3((unsigned)blocks), dim3(threads1(ctx)), args1,
-                                       (size_t)budget, ctx->stream);
+    const int variant = variant1(ctx, n);   // (its limits were set by the eager step of the same key)
+    int threads = 0;
+    bool fits = false;
+    if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
+    if (!fits) return cudaErrorCooperativeLaunchTooLarge;
+    return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, (size_t)budget,
+                                       ctx->stream);
 }
 
 cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)

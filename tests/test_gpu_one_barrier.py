@@ -121,3 +121,19 @@ def test_shapes_in_turn_on_one_context():
     for shape, x in zip(shapes, got):
         with A.Context(params, s.n, 12 * s.n) as ctx:
             assert np.array_equal(one(ctx, *shape), x)
+
+
+@pytest.mark.parametrize("shape", [(768, 0), (1024, 0)])
+def test_recorded_step_repeats_the_eager_one(shape):
+    s = system(20000)   # past the line between the kernels with and without the barrier
+    with A.Context(A.params_of(s, precision=A.MIXED, tol=1e-6), s.n, 12 * s.n) as ctx:
+        ctx.set_launch(*shape)
+        ctx.set_step_graph(True)
+        x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+        got = []
+        for _ in range(4):   # eager, recorded, replayed twice
+            x.copy_(dev(s.x))
+            q.copy_(dev(s.quat))
+            assert ctx.step(x, q, f).solver == SOLVER_ONE
+            got.append(host(x).copy())
+    assert all(np.array_equal(got[0], g) for g in got[1:])
