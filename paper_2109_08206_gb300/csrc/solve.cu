@@ -3591,6 +3591,67 @@ static cudaError_t ready1(aLENS_ctx* ctx, int variant, size_t budget, int& threa
     return cudaSuccess;
 }
 
+// Dynamic shared memory that a block may ask for where its SM (bps blocks)
+// divides its 256 KB into kb KB of shared memory and the rest of L1 (1 KB a
+// block is the system's).
+template <typename T>
+static long long dyn_within(const aLENS_ctx* ctx, int kb)
+{
+    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
+    return (long long)(kb / bps) * 1024 - (long long)sizeof(Shared1<T>) - 1024;
+}
+
+// Dynamic shared memory of a one-barrier launch whose largest share needs
+// `need` bytes: the share proper, with room for ds and gs (2 values for 13)
+// and for a halo rod (6 values) per slot, but no more than leaves the L1 that
+// the share itself leaves, up to 92 KB of it: the kernel's spilled registers
+// live there, and where the largest division leaves 28 KB they go to L2 (the
+// steps of the division are the device's).  Solve, ms, with the whole room
+// and so: 3e4 rods float64 7.86 / 5.20, 1.6e4 rods float64 in caller order
+// 8.22 / 4.87, 3e4 rods float64 at 512 x 2 11.5 / 8.45, 6e4 rods mixed 2.14 /
+// 1.91; a halo that finds no room then is polled slot by slot.
+template <typename T>
+static long long request1(const aLENS_ctx* ctx, long long need, long long budget)
+{
+    long long room = need + need * 8 / 13;
+    for (int kb : {164, 196}) {
+        const long long most = dyn_within<T>(ctx, kb);
+        if (need <= most) {
+            if (room > most) room = most;
+            break;
+        }
+    }
+    return room < budget ? room : budget;
+}
+
+// Cooperative launch of a one-barrier kernel with the SM divided for the bps
+// blocks that it holds: left alone, the driver divides it for as many as their
+// registers allow, which leaves less L1 (2e4 rods at 256 x 1 mixed 0.86 ms /
+// 0.70 so, at 256 x 3 float64 7.30 / 5.36).
+template <typename T>
+static cudaError_t launch1(const aLENS_ctx* ctx, int variant, int blocks, int threads, SolveArgs<T>& a)
+{
+    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
+    const size_t total = (size_t)bps * (a.dyn_bytes + sizeof(Shared1<T>) + 1024);
+    int kb = 228;
+    for (int k : {196, 164, 132, 100, 64, 32, 16, 8})
+        if (total <= (size_t)k * 1024) kb = k;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[1].val.sharedMemCarveout = (unsigned)(100 * kb / 228);   // (rounded up to the next division)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = a.dyn_bytes;
+    cfg.stream = ctx->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    void* args[] = {&a};
+    return cudaLaunchKernelExC(&cfg, kernel1<T>(variant), args);
+}
+
 template <typename T>
 static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, int m)
 {
@@ -3631,15 +3692,10 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
         bool fits = false;
         if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
         if (fits && (long long)bps * ctx->num_sms >= blocks) {
-            // the share proper, with room for ds and gs (2 values for 13) and for
-            // a halo rod (6 values) per slot
-            const long long room = (long long)need1 + (long long)need1 * 8 / 13;
-            a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : room < budget ? room : budget);
-            void* args1[] = {&a};
+            a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : request1<T>(ctx, (long long)need1, budget));
             ++ctx->launches;
             ctx->last_solver = 1;
-            return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, a.dyn_bytes,
-                                               ctx->stream);
+            return launch1<T>(ctx, variant, (int)blocks, threads, a);
         }
     }
     if ((e = launch_setup_qe(ctx)) != cudaSuccess) return e;   // the two-barrier kernels read qe
@@ -3825,7 +3881,6 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
                                                              ctx->dcount + C_MAXRODS, ctx->dcount + C_SMEM1);
     ++ctx->launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
     const int variant = variant1(ctx, n);   // (its limits were set by the eager step of the same key)
@@ -3833,8 +3888,7 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     bool fits = false;
     if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
     if (!fits) return cudaErrorCooperativeLaunchTooLarge;
-    return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, (size_t)budget,
-                                       ctx->stream);
+    return launch1<T>(ctx, variant, (int)blocks, threads, a);
 }
 
 cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)

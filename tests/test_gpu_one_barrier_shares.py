@@ -1,0 +1,46 @@
+"""The one-barrier solver's launches: kernel, shared memory and what they cost."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2109_08206_gb300 as A  # noqa: E402
+
+from test_gpu_one_barrier import SOLVER_ONE, SOLVERS_TWO, system  # noqa: E402
+from test_gpu_parity import dev  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+TOL = {A.FP64: 1e-6, A.MIXED: 1e-5}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    A.build()
+    assert torch.cuda.is_available()
+
+
+def us_per_iteration(call, repeats=7):
+    """Least solve time per iteration over the repeats, and the last call's info."""
+    infos = [call() for _ in range(repeats)]
+    return min(i.ms_solve for i in infos) * 1e3 / infos[-1].iters, infos[-1]
+
+
+def timed_lcp(s, precision, barriers=1):
+    with A.Context(A.params_of(s, precision=precision, tol=TOL[precision]), s.n, 12 * s.n) as ctx:
+        ctx.set_solver_schedule(barriers)
+        x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+        pairs = ctx.build_neighbors(x, q)
+        _, dgeom, lq = ctx.assemble_constraints(x, q, f, pairs)
+        return us_per_iteration(lambda: ctx.solve_lcp(q, pairs, dgeom, lq)[1])
+
+
+def test_float64_shares_leave_l1_for_the_spills():
+    """An iteration of the one-barrier solver is no longer than one of the
+    two-barrier schedule it stands in for (a tenth for the clock): where the
+    launch took all the shared memory, the registers that the kernel spills
+    went to L2 and this one was half as long again."""
+    s = system(16000, phi=0.10)
+    one, info = timed_lcp(s, A.FP64)
+    two, info2 = timed_lcp(s, A.FP64, barriers=2)
+    assert info.solver == SOLVER_ONE and info2.solver in SOLVERS_TWO
+    assert one <= 1.1 * two, (one, two)
