@@ -3624,34 +3624,6 @@ static long long request1(const aLENS_ctx* ctx, long long need, long long budget
     return room < budget ? room : budget;
 }
 
-// Cooperative launch of a one-barrier kernel with the SM divided for the bps
-// blocks that it holds: left alone, the driver divides it for as many as their
-// registers allow, which leaves less L1 (2e4 rods at 256 x 1 mixed 0.86 ms /
-// 0.70 so, at 256 x 3 float64 7.30 / 5.36).
-template <typename T>
-static cudaError_t launch1(const aLENS_ctx* ctx, int variant, int blocks, int threads, SolveArgs<T>& a)
-{
-    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
-    const size_t total = (size_t)bps * (a.dyn_bytes + sizeof(Shared1<T>) + 1024);
-    int kb = 228;
-    for (int k : {196, 164, 132, 100, 64, 32, 16, 8})
-        if (total <= (size_t)k * 1024) kb = k;
-    cudaLaunchAttribute at[2] = {};
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    at[1].val.sharedMemCarveout = (unsigned)(100 * kb / 228);   // (rounded up to the next division)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = a.dyn_bytes;
-    cfg.stream = ctx->stream;
-    cfg.attrs = at;
-    cfg.numAttrs = 2;
-    void* args[] = {&a};
-    return cudaLaunchKernelExC(&cfg, kernel1<T>(variant), args);
-}
-
 template <typename T>
 static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, int m)
 {
@@ -3693,9 +3665,11 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
         if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
         if (fits && (long long)bps * ctx->num_sms >= blocks) {
             a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : request1<T>(ctx, (long long)need1, budget));
+            void* args1[] = {&a};
             ++ctx->launches;
             ctx->last_solver = 1;
-            return launch1<T>(ctx, variant, (int)blocks, threads, a);
+            return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, a.dyn_bytes,
+                                               ctx->stream);
         }
     }
     if ((e = launch_setup_qe(ctx)) != cudaSuccess) return e;   // the two-barrier kernels read qe
@@ -3881,6 +3855,7 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
                                                              ctx->dcount + C_MAXRODS, ctx->dcount + C_SMEM1);
     ++ctx->launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
     const int variant = variant1(ctx, n);   // (its limits were set by the eager step of the same key)
@@ -3888,7 +3863,8 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     bool fits = false;
     if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
     if (!fits) return cudaErrorCooperativeLaunchTooLarge;
-    return launch1<T>(ctx, variant, (int)blocks, threads, a);
+    return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, a.dyn_bytes,
+                                       ctx->stream);
 }
 
 cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)

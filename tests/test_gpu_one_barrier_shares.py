@@ -25,6 +25,21 @@ def us_per_iteration(call, repeats=7):
     return min(i.ms_solve for i in infos) * 1e3 / infos[-1].iters, infos[-1]
 
 
+def timed_step(s, precision, threads, bps, barriers=1):
+    with A.Context(A.params_of(s, precision=precision, tol=TOL[precision]), s.n, 12 * s.n) as ctx:
+        ctx.set_launch(threads, bps)
+        ctx.set_solver_schedule(barriers)
+        x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+        x0, q0 = x.clone(), q.clone()
+
+        def call():
+            x.copy_(x0)
+            q.copy_(q0)
+            return ctx.step(x, q, f)
+
+        return us_per_iteration(call)
+
+
 def timed_lcp(s, precision, barriers=1):
     with A.Context(A.params_of(s, precision=precision, tol=TOL[precision]), s.n, 12 * s.n) as ctx:
         ctx.set_solver_schedule(barriers)
@@ -42,5 +57,15 @@ def test_float64_shares_leave_l1_for_the_spills():
     s = system(16000, phi=0.10)
     one, info = timed_lcp(s, A.FP64)
     two, info2 = timed_lcp(s, A.FP64, barriers=2)
+    assert info.solver == SOLVER_ONE and info2.solver in SOLVERS_TWO
+    assert one <= 1.1 * two, (one, two)
+
+
+def test_shares_that_fill_an_sm_of_several_blocks_meet_at_a_barrier():
+    """The same bound: here the share itself leaves no L1, and the kernel without
+    spills is the faster one."""
+    s = system(50000, phi=0.10)
+    one, info = timed_step(s, A.MIXED, 256, 4)
+    two, info2 = timed_step(s, A.MIXED, 256, 4, barriers=2)
     assert info.solver == SOLVER_ONE and info2.solver in SOLVERS_TWO
     assert one <= 1.1 * two, (one, two)
