@@ -385,6 +385,7 @@ struct aLENS_ctx {
     int attr1_set[2];        // the one-barrier kernels' dynamic shared-memory limits that are set (a bit each; float, double)
     int occ1_key[2];         // kernel and launch shape whose occupancy was checked ...
     int occ1_ok[2];          // ... and whether that many blocks per SM fit at the full budget
+    int occ1_regs[2];        // ... and how many fit by their registers
     int last_solver;         // kernel of the last single-system solve: 1 one-barrier, 2 two-barrier staged, 3 two-barrier global
     int zero_start;          // the last setup started from gamma = 0 (no caller gamma)
     int caller_order;        // the last layout took the rods in the caller's order (no rank)

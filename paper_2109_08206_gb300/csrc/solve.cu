@@ -64,6 +64,7 @@
 #include <cooperative_groups.h>
 #include <float.h>
 
+#include <algorithm>
 #include <cmath>
 #include <limits>
 #include <type_traits>
@@ -3547,16 +3548,41 @@ static int threads1(const aLENS_ctx* ctx)
 
 static_assert(sizeof(Shared1<double>) <= sizeof(Shared<double>) + 768 && sizeof(Shared1<float>) <= sizeof(Shared<float>) + 768,
               "the one-barrier kernel's static shared memory and the shares' budget exceed a block's limit");
-// The one-barrier kernel of a launch: with the barrier for large systems in
-// caller order or with 1024 workers (no room for a warp of the sums' own: 1e5
-// rods 10.8 us an iteration against 13.3), without it in the default shape (72
-// registers a thread) and in the others (several blocks on an SM share its
-// registers).
-enum { V_MEET = 0, V_WIDE = 1, V_ANY = 2 };
-static int variant1(const aLENS_ctx* ctx, int n)
+// Dynamic shared memory that a block may ask for where `blocks` of them share an
+// SM that divides its 256 KB into kb KB of shared memory and the rest of L1
+// (1 KB a block is the system's, and one is left free).
+template <typename T>
+static long long dyn_within(int kb, int blocks)
 {
-    if ((ctx->caller_order || (ctx->solve_threads > 992 && ctx->solve_bps <= 1)) && n > kMeetRods) return V_MEET;
-    return threads1(ctx) <= kThreads1 && ctx->solve_bps <= 1 ? V_WIDE : V_ANY;
+    return (long long)(kb / blocks) * 1024 - (long long)sizeof(Shared1<T>) - 2048;
+}
+
+// The one-barrier kernel of a launch whose largest share needs `need` bytes.
+// With the barrier:
+//  - above kMeetRods rods in caller order, or with 1024 workers (no room for a
+//    warp of the sums' own: 1e5 rods 10.8 us an iteration against 13.3);
+//  - where the other one has 64 registers a thread (every shape but up to 768
+//    workers one block an SM) and the share leaves too little L1 for what it
+//    spills: 576 bytes a thread in float64, 204 in float32 (solve, ms, barrier /
+//    tagged: 4.5e4 rods float64 at 992 x 1 7.90 / 8.81, 4e4 at 512 x 2 6.63 /
+//    8.77, 2e4 at 256 x 3 5.96 / 7.31; mixed 5e4 rods at 256 x 4 1.84 / 5.91,
+//    1e4 dense ones 5.2 / 7.3);
+//  - several blocks an SM, above 10,000 rods in float32: as every block reads
+//    every block's sums, and the halo grows with the blocks (1.0e4 rods at 512 x
+//    2 and 256 x 4 0.91 / 0.91 and 0.88 / 0.87, 1.2e4 1.18 / 1.18 and 1.02 /
+//    1.04, 3e4 1.44 / 1.47 and 1.93 / 2.45).
+// Without it elsewhere, with 80 registers a thread in the default shape.
+enum { V_MEET = 0, V_WIDE = 1, V_ANY = 2 };
+constexpr int kMeetRodsSeveral = 10000;
+template <typename T>
+static int variant1(const aLENS_ctx* ctx, int n, long long need)
+{
+    const bool several = ctx->solve_bps > 1;
+    if ((ctx->caller_order || (ctx->solve_threads > 992 && !several)) && n > kMeetRods) return V_MEET;
+    if (threads1(ctx) <= kThreads1 && !several) return V_WIDE;
+    const bool f32 = sizeof(T) == 4;
+    if (need > dyn_within<T>(f32 ? 196 : 164, several ? ctx->solve_bps : 1) || (f32 && several && n > kMeetRodsSeveral)) return V_MEET;
+    return V_ANY;
 }
 template <typename T>
 static const void* kernel1(int variant)
@@ -3585,20 +3611,11 @@ static cudaError_t ready1(aLENS_ctx* ctx, int variant, size_t budget, int& threa
         int per_sm = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, budget)) != cudaSuccess) return e;
         ctx->occ1_ok[ti] = per_sm >= bps;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->occ1_regs[ti], fn, threads, 0)) != cudaSuccess) return e;
         ctx->occ1_key[ti] = key;
     }
     fits = ctx->occ1_ok[ti] != 0;
     return cudaSuccess;
-}
-
-// Dynamic shared memory that a block may ask for where its SM (bps blocks)
-// divides its 256 KB into kb KB of shared memory and the rest of L1 (1 KB a
-// block is the system's).
-template <typename T>
-static long long dyn_within(const aLENS_ctx* ctx, int kb)
-{
-    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
-    return (long long)(kb / bps) * 1024 - (long long)sizeof(Shared1<T>) - 1024;
 }
 
 // Dynamic shared memory of a one-barrier launch whose largest share needs
@@ -3610,16 +3627,19 @@ static long long dyn_within(const aLENS_ctx* ctx, int kb)
 // and so: 3e4 rods float64 7.86 / 5.20, 1.6e4 rods float64 in caller order
 // 8.22 / 4.87, 3e4 rods float64 at 512 x 2 11.5 / 8.45, 6e4 rods mixed 2.14 /
 // 1.91; a halo that finds no room then is polled slot by slot.
+// The driver divides an SM for as many blocks as their registers allow
+// (by_regs), so a launch of fewer asks for little enough that all those fit
+// the division, or for too much for one more than bps.
 template <typename T>
-static long long request1(const aLENS_ctx* ctx, long long need, long long budget)
+static long long request1(const aLENS_ctx* ctx, int by_regs, long long need, long long budget)
 {
-    long long room = need + need * 8 / 13;
+    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
+    const long long room = need + need * 8 / 13;
     for (int kb : {164, 196}) {
-        const long long most = dyn_within<T>(ctx, kb);
-        if (need <= most) {
-            if (room > most) room = most;
-            break;
-        }
+        const long long all = dyn_within<T>(kb, by_regs), most = dyn_within<T>(kb, bps);
+        if (need <= all) return room < all ? room : all;
+        const long long least = std::max(need, 228ll * 1024 / (bps + 1));
+        if (by_regs > bps && least <= most) return std::min(std::max(room, least), most);
     }
     return room < budget ? room : budget;
 }
@@ -3659,12 +3679,12 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
     const long long budget = (long long)optin / bps - (long long)sizeof(Shared<T>) - 1024;
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
         // at most one grid barrier per iteration: every block's share and its ghosts fit
-        const int variant = variant1(ctx, n);
+        const int variant = variant1<T>(ctx, n, (long long)need1);
         int threads = 0;
         bool fits = false;
         if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
         if (fits && (long long)bps * ctx->num_sms >= blocks) {
-            a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : request1<T>(ctx, (long long)need1, budget));
+            a.dyn_bytes = (size_t)(variant == V_MEET ? (long long)need1 : request1<T>(ctx, ctx->occ1_regs[sizeof(T) == 4 ? 0 : 1], (long long)need1, budget));
             void* args1[] = {&a};
             ++ctx->launches;
             ctx->last_solver = 1;
@@ -3831,7 +3851,7 @@ static cudaError_t graph1_check(aLENS_ctx* ctx, bool& ok)
     ok = false;
     if (ctx->solve_barriers != 1 || ctx->solve_threads < 256) return cudaSuccess;
     int threads = 0;
-    return ready1<T>(ctx, variant1(ctx, 0), (size_t)graph1_budget<T>(ctx), threads, ok);
+    return ready1<T>(ctx, variant1<T>(ctx, 0, 0), (size_t)graph1_budget<T>(ctx), threads, ok);
 }
 
 template <typename T>
@@ -3858,7 +3878,7 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
-    const int variant = variant1(ctx, n);   // (its limits were set by the eager step of the same key)
+    const int variant = variant1<T>(ctx, n, 0);   // (its limits were set by the eager step of the same key)
     int threads = 0;
     bool fits = false;
     if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
