@@ -985,8 +985,10 @@ static aLENS_status step_batch_graph(aLENS_ctx* c, int64_t n, double* x, double*
 
 // The same for a single-system step: the first step of a key runs eagerly
 // (ALENS_ERR_NOT_IMPLEMENTED), and a key whose eager step did not run the
-// one-barrier solver, or whose replay found a share too big for the
-// recorded launch (kSolveRedo: nothing moved), stays eager.
+// one-barrier solver stays eager.  A replay that finds a share too big for
+// the recorded launch (kSolveRedo: nothing moved) runs eagerly, and the next
+// step is recorded anew with room for that share; a launch that had asked for
+// all the shared memory there is leaves the key eager.
 static aLENS_status step_single_graph(aLENS_ctx* c, int64_t n, double* x, double* quat, const double* f_nc,
                                       int32_t* pairs_out, double* gamma_out, double* vel_out, aLENS_info* info)
 {
@@ -1001,7 +1003,7 @@ static aLENS_status step_single_graph(aLENS_ctx* c, int64_t n, double* x, double
     if (c->graph_state == 3) return ALENS_ERR_NOT_IMPLEMENTED;
     if (c->graph_state == 1) {
         bool ok = false;
-        CK(graph1_possible(c, c->p.precision, ok));
+        CK(graph1_possible(c, (int)n, c->p.precision, ok));
         if (!ok) {
             c->graph_state = 3;
             return ALENS_ERR_NOT_IMPLEMENTED;
@@ -1017,7 +1019,7 @@ static aLENS_status step_single_graph(aLENS_ctx* c, int64_t n, double* x, double
     if (c->hflags[F_SOLVE_ERR] == kSolveRedo) {
         drop_graph(c);
         c->gkey = k;
-        c->graph_state = 3;
+        c->graph_state = c->graph_full ? 3 : 1;
         return ALENS_ERR_NOT_IMPLEMENTED;
     }
     return graph_outcome(c, n, info);
@@ -1038,8 +1040,10 @@ aLENS_status aLENS_step(aLENS_ctx* c, int64_t n, double* x, double* quat, const 
     if (st != ALENS_ERR_NOT_IMPLEMENTED) return st;
     c->launches = 0;
     st = step_impl(c, n, x, quat, f_nc, pairs_out, gamma_out, vel_out, info);
-    // a key whose eager step did not run the one-barrier solver stays eager
-    if (graphable && c->graph_state == 1 && c->last_solver != 1) c->graph_state = 3;
+    if (graphable && c->graph_state == 1) {
+        if (c->last_solver != 1) c->graph_state = 3;   // a key whose eager step did not run the one-barrier solver stays eager
+        else c->graph_need = c->last_need1;
+    }
     return st;
 }
 

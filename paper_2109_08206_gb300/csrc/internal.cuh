@@ -386,6 +386,9 @@ struct aLENS_ctx {
     int occ1_key[2];         // kernel and launch shape whose occupancy was checked ...
     int occ1_ok[2];          // ... and whether that many blocks per SM fit at the full budget
     int occ1_regs[2];        // ... and how many fit by their registers
+    unsigned long long last_need1;   // largest one-barrier share of the last single-system solve (bytes)
+    unsigned long long graph_need;   // ... of the eager step of the recorded step's key
+    int graph_full;          // the recorded solve asked for all the shared memory a block may ask for
     int last_solver;         // kernel of the last single-system solve: 1 one-barrier, 2 two-barrier staged, 3 two-barrier global
     int zero_start;          // the last setup started from gamma = 0 (no caller gamma)
     int caller_order;        // the last layout took the rods in the caller's order (no rank)
@@ -508,7 +511,7 @@ cudaError_t launch_setup_qe(aLENS_ctx* ctx);
 // kernel checks on the device that its shares fit and otherwise flags
 // kSolveRedo), and whether the context's launch shape allows it.
 cudaError_t launch_solve_graph1(aLENS_ctx* ctx, int n, int m, int precision);
-cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok);
+cudaError_t graph1_possible(aLENS_ctx* ctx, int n, int precision, bool& ok);
 cudaError_t launch_gamma_out(aLENS_ctx* ctx, int m, int precision, double* gamma_out);
 
 // Springs: rows mu .. mu + nb of the internal constraint list (pairs, phi,

@@ -3675,6 +3675,7 @@ static cudaError_t solve_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, int n, in
         (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess)
         return e;
     const unsigned long long need = hb[0], maxrods = hb[C_MAXRODS - C_SMEM], need1 = hb[C_SMEM1 - C_SMEM];
+    ctx->last_need1 = need1;
     const int optin = ctx->smem_optin;
     const long long budget = (long long)optin / bps - (long long)sizeof(Shared<T>) - 1024;
     if (ctx->solve_barriers == 1 && threads >= 256 && need1 > 0 && (long long)need1 <= budget) {
@@ -3831,27 +3832,39 @@ cudaError_t launch_solve(aLENS_ctx* ctx, int n, int m, int precision)
 }
 
 // The single-system solve of a step recorded as a CUDA graph: no readback.
-// The one-barrier kernel is launched with the full shared-memory budget of
-// the launch shape, and its blocks check the need of the shares (computed
-// on the device by k_shares) against it: a share that does not fit
-// makes every block leave before its first barrier with kSolveRedo in
-// F_SOLVE_ERR, the update and the outputs then leave everything untouched,
-// and the caller runs the step eagerly.  graph1_possible says whether the
-// launch shape can take this path at all.
+// The kernel and its shared memory are chosen for the largest share of the
+// eager step of the same key (graph_need), and its blocks check the need of
+// the shares (computed on the device by k_shares) against it: a share that
+// does not fit makes every block leave before its first barrier with
+// kSolveRedo in F_SOLVE_ERR, the update and the outputs then leave everything
+// untouched, and the caller runs the step eagerly.  (With all the shared
+// memory a block may ask for, little L1 is left for the kernel's spills:
+// 2e4 rods float64 4.13 ms against 2.98, 1e4 rods mixed at 256 x 4 1.65
+// against 0.87.)
 template <typename T>
-static long long graph1_budget(const aLENS_ctx* ctx)
-{
-    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
-    return (long long)ctx->smem_optin / bps - (long long)sizeof(Shared<T>) - 1024;
-}
-
-template <typename T>
-static cudaError_t graph1_check(aLENS_ctx* ctx, bool& ok)
+static cudaError_t plan_graph1(aLENS_ctx* ctx, int n, SolveArgs<T>* a, int& variant, int& threads, bool& ok)
 {
     ok = false;
     if (ctx->solve_barriers != 1 || ctx->solve_threads < 256) return cudaSuccess;
-    int threads = 0;
-    return ready1<T>(ctx, variant1<T>(ctx, 0, 0), (size_t)graph1_budget<T>(ctx), threads, ok);
+    const int bps = ctx->solve_bps > 0 ? ctx->solve_bps : 1;
+    const long long budget = (long long)ctx->smem_optin / bps - (long long)sizeof(Shared<T>) - 1024;
+    const long long need = (long long)ctx->graph_need;
+    variant = variant1<T>(ctx, n, need);
+    const cudaError_t e = ready1<T>(ctx, variant, (size_t)budget, threads, ok);
+    if (a && e == cudaSuccess) {
+        a->dyn_bytes = (size_t)request1<T>(ctx, ctx->occ1_regs[sizeof(T) == 4 ? 0 : 1], need, budget);
+        a->fit_cap = (long long)a->dyn_bytes;
+        ctx->graph_full = (long long)a->dyn_bytes >= budget;
+    }
+    return e;
+}
+
+template <typename T>
+static cudaError_t graph1_check(aLENS_ctx* ctx, int n, bool& ok)
+{
+    int variant = 0, threads = 0;
+    ctx->caller_order = 0;   // (a step's: the layout sets it, which is not yet recorded)
+    return plan_graph1<T>(ctx, n, nullptr, variant, threads, ok);
 }
 
 template <typename T>
@@ -3865,11 +3878,16 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     long long blocks = (long long)bps * ctx->num_sms;
     if (want < blocks) blocks = want < 1 ? 1 : want;
     if (blocks > ctx->max_blocks) blocks = ctx->max_blocks;
-    const long long budget = graph1_budget<T>(ctx);
+    int variant = 0, threads = 0;
+    bool fits = false;
+    cudaError_t e = plan_graph1<T>(ctx, n, &a, variant, threads, fits);
+    if (e != cudaSuccess) return e;
+    if (!fits) return cudaErrorCooperativeLaunchTooLarge;
     a.need1_dev = ctx->dcount + C_SMEM1;
-    a.fit_cap = force_redo ? 0 : budget;
-    a.dyn_bytes = (size_t)budget;
-    cudaError_t e;
+    if (force_redo) {
+        a.fit_cap = 0;
+        ctx->graph_full = 1;
+    }
     k_shares<<<(int)blocks, kNeedThreads, 0, ctx->stream>>>(n, (int)blocks, (int)sizeof(T), ctx->rowP, ctx->rowQ, ctx->qlist,
                                                              ctx->bstart, ctx->bar, ctx->dcount + C_SMEM,
                                                              ctx->dcount + C_MAXRODS, ctx->dcount + C_SMEM1);
@@ -3878,18 +3896,14 @@ static cudaError_t solve_graph1_typed(aLENS_ctx* ctx, const SolveBufs<T>& sb, in
     void* args1[] = {&a};
     ++ctx->launches;
     ctx->last_solver = 1;
-    const int variant = variant1<T>(ctx, n, 0);   // (its limits were set by the eager step of the same key)
-    int threads = 0;
-    bool fits = false;
-    if ((e = ready1<T>(ctx, variant, (size_t)budget, threads, fits)) != cudaSuccess) return e;
-    if (!fits) return cudaErrorCooperativeLaunchTooLarge;
     return cudaLaunchCooperativeKernel(kernel1<T>(variant), dim3((unsigned)blocks), dim3(threads), args1, a.dyn_bytes,
                                        ctx->stream);
 }
 
-cudaError_t graph1_possible(aLENS_ctx* ctx, int precision, bool& ok)
+// Whether the launch that would be recorded fits the device at all.
+cudaError_t graph1_possible(aLENS_ctx* ctx, int n, int precision, bool& ok)
 {
-    return precision == ALENS_MIXED ? graph1_check<float>(ctx, ok) : graph1_check<double>(ctx, ok);
+    return precision == ALENS_MIXED ? graph1_check<float>(ctx, n, ok) : graph1_check<double>(ctx, n, ok);
 }
 
 cudaError_t launch_solve_graph1(aLENS_ctx* ctx, int n, int m, int precision)

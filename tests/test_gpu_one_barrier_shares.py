@@ -25,10 +25,11 @@ def us_per_iteration(call, repeats=7):
     return min(i.ms_solve for i in infos) * 1e3 / infos[-1].iters, infos[-1]
 
 
-def timed_step(s, precision, threads, bps, barriers=1):
+def timed_step(s, precision, threads, bps, barriers=1, graph=False):
     with A.Context(A.params_of(s, precision=precision, tol=TOL[precision]), s.n, 12 * s.n) as ctx:
         ctx.set_launch(threads, bps)
         ctx.set_solver_schedule(barriers)
+        ctx.set_step_graph(graph)
         x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
         x0, q0 = x.clone(), q.clone()
 
@@ -37,6 +38,8 @@ def timed_step(s, precision, threads, bps, barriers=1):
             q.copy_(q0)
             return ctx.step(x, q, f)
 
+        if graph:
+            call(), call()   # eager, recorded
         return us_per_iteration(call)
 
 
@@ -69,3 +72,45 @@ def test_shares_that_fill_an_sm_of_several_blocks_meet_at_a_barrier():
     two, info2 = timed_step(s, A.MIXED, 256, 4, barriers=2)
     assert info.solver == SOLVER_ONE and info2.solver in SOLVERS_TWO
     assert one <= 1.1 * two, (one, two)
+
+
+def test_recorded_step_asks_for_the_eager_steps_shared_memory():
+    """The recorded solve is the eager one (a quarter for the clock and for what
+    runs beside it)."""
+    s = system(10000, phi=0.10)
+    eager, info = timed_step(s, A.MIXED, 256, 4)
+    recorded, info2 = timed_step(s, A.MIXED, 256, 4, graph=True)
+    assert info.solver == info2.solver == SOLVER_ONE and info.iters == info2.iters
+    assert recorded <= 1.25 * eager, (recorded, eager)
+
+
+@pytest.mark.parametrize("precision", [A.FP64, A.MIXED])
+def test_recorded_step_outgrown_by_its_shares(precision):
+    """Rods that close in until their shares no longer fit what the recorded
+    step asked for: that step runs eagerly, the next is recorded anew, and all of
+    them give what eager steps give, on the way back as well."""
+    s = system(3000)
+    scales = [1.0, 1.0, 1.0, 0.6, 0.6, 0.6, 0.6, 1.0]
+    got = []
+    for graph in (False, True):
+        with A.Context(A.params_of(s, precision=precision, tol=TOL[precision], max_iter=1_000_000), s.n, 64 * s.n) as ctx:
+            ctx.set_step_graph(graph)
+            x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+            x0, q0 = x.clone(), q.clone()
+            out = []
+            for scale in scales:
+                x.copy_(x0 * scale)
+                q.copy_(q0)
+                info = ctx.step(x, q, f)
+                assert info.solver == SOLVER_ONE
+                out.append((info, x.clone(), q.clone()))
+            got.append(out)
+    eager, recorded = got
+    assert eager[3][0].n_pairs > 3 * eager[0][0].n_pairs
+    for (a, xa, qa), (b, xb, qb) in zip(eager, recorded):
+        assert (a.n_pairs, a.iters, a.residual) == (b.n_pairs, b.iters, b.residual)
+        assert torch.equal(xa, xb) and torch.equal(qa, qb)
+    launches = [info.launches for info, _, _ in recorded]
+    replay, plain = launches[2], eager[2][0].launches
+    assert replay != plain
+    assert launches == [plain, replay, replay, plain, replay, replay, replay, replay]
