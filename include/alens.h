@@ -438,8 +438,10 @@ ALENS_API aLENS_status aLENS_set_scaling(aLENS_ctx* ctx, double beta);
  * that the first cluster's bounded waits run out.  mode 2 makes the next
  * recorded single-system step (aLENS_set_step_graph) find its shares too
  * big for its launch, so that the call falls back to a step without a
- * graph.  These clear themselves after one launch or recording; mode 0
- * disables them.  mode 3 makes the context's batched solver run as on a
+ * graph.  mode 4 is mode 1 after the first grid barrier of the single-system
+ * one-barrier solver, so that the waits for that block's velocities and
+ * sums run out.  These clear themselves after one launch or recording; mode
+ * 0 disables them.  mode 3 makes the context's batched solver run as on a
  * device that refuses a cooperative launch with clusters: every system is
  * solved by one cluster from then on (drops a recorded batched step). */
 ALENS_API aLENS_status aLENS_inject_fault(aLENS_ctx* ctx, int32_t mode);

@@ -548,7 +548,7 @@ static void drop_graph(aLENS_ctx* c);
 
 aLENS_status aLENS_inject_fault(aLENS_ctx* c, int32_t mode)
 {
-    if (!c || mode < 0 || mode > 3) return ALENS_ERR_INVALID;
+    if (!c || mode < 0 || mode > 4) return ALENS_ERR_INVALID;
     if (mode == 3) {   // as after a refused cooperative cluster launch: no pairs from now on
         c->batch_coop = 0;
         drop_graph(c);
@@ -1033,8 +1033,9 @@ aLENS_status aLENS_step(aLENS_ctx* c, int64_t n, double* x, double* quat, const 
     if (c) { c->launches = 0; c->last_solver = 0; single_mode(c); }
     if (!rods_ok(c, n) || (n > 0 && (!x || !quat))) return ALENS_ERR_INVALID;
     if (!c->coop_ok) return ALENS_ERR_CUDA;
-    // graph mode: plain steps (no springs, walls or bounded-wait test hook)
-    const bool graphable = c->step_graph && n > 0 && c->sp_n == 0 && c->wall_axis < 0 && c->fault_mode != 1;
+    // graph mode: plain steps (no springs, walls or bounded-wait test hooks)
+    const bool graphable = c->step_graph && n > 0 && c->sp_n == 0 && c->wall_axis < 0 && c->fault_mode != 1 &&
+                           c->fault_mode != 4;
     aLENS_status st = ALENS_ERR_NOT_IMPLEMENTED;
     if (graphable) st = step_single_graph(c, n, x, quat, f_nc, pairs_out, gamma_out, vel_out, info);
     if (st != ALENS_ERR_NOT_IMPLEMENTED) return st;

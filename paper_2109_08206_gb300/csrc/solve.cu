@@ -1593,7 +1593,10 @@ struct Shared1 {
     int kind, ng, nh, ne;
     int nref;               // refreshes taken: the reference lives in state buffer nref & 1
     unsigned epoch;         // grid barriers passed (thread 0's)
-    int bad;    // a wait ran out (or another block's did): the block leaves
+    // a wait ran out (or another block's did): the block leaves.  One word for the waits
+    // of the constraint phase and one for those after it, each read by every
+    // thread between block barriers that no write to it crosses.
+    int bad[2];
 };
 
 template <typename T> struct Row { T x, y, z, w; };
@@ -2351,7 +2354,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
         o.q1 = a.rowQ[o.r1];
         o.nc = o.c1 - o.c0;
         o.cap_r = o.r1 - o.r0;
-        sh.bad = 0;
+        sh.bad[0] = sh.bad[1] = 0;
         sh.alpha0 = T(1);
         sh.pimax = T(0);
         sh.k = sh.since = sh.hist = sh.nref = 0;
@@ -2413,6 +2416,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
         __syncthreads();   // red is read
         sort_rods_total(o, reinterpret_cast<int*>(sh.red));
         if (!barrier()) return;
+        if (a.fault == 4 && blockIdx.x == 0) return;   // test hook: its words never come
         if (duty) {
             T tot[4] = {T(0), T(0), T(0), T(0)};
             for (int b = lane; b < nb; b += 32) {
@@ -2459,8 +2463,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
                 v[3] = s3;
                 cpub = C_REF1;
             } else {
-                if (o.halo) con_pass_step1<T, false>(a, o, sh.alpha, xr, tag, &sh.bad, v);
-                else con_pass_step1<T, true>(a, o, sh.alpha, xr, tag, &sh.bad, v);
+                if (o.halo) con_pass_step1<T, false>(a, o, sh.alpha, xr, tag, &sh.bad[0], v);
+                else con_pass_step1<T, true>(a, o, sh.alpha, xr, tag, &sh.bad[0], v);
                 cpub = C_STEP1;
             }
             if ((int)threadIdx.x < a.workers) {
@@ -2469,7 +2473,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
                 else if ((threadIdx.x & 31) < 4) sh.red[threadIdx.x >> 5][threadIdx.x & 3] = T(0);
             }
             __syncthreads();
-            if (sh.bad) return;
+            if (sh.bad[0]) return;
+        } else {
+            __syncthreads();   // sh.kind is read before the first decision replaces it
         }
         ++tag;
         if (duty && cpub != C_NONE1) {   // this block's sums, while the others run the rod phase
@@ -2480,14 +2486,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
         uint4* const xw = a.xch + (tag & 1u) * (Xch<T>::kWords * (size_t)a.n);
         if (8 * (o.r1 - o.r0) <= a.workers) rod_step8(a, o, xw, tag);
         else rod_step2(a, o, xw, tag);
-        fetch_halo(a, o, xw, tag, &sh.bad);
+        fetch_halo(a, o, xw, tag, &sh.bad[1]);
         if (duty) {   // the next iteration's step
             T tot[4];
-            if (cpub != C_NONE1) grid_sums1(a, sums(tag), (int)gridDim.x, tag, &sh.bad, tot);
+            if (cpub != C_NONE1) grid_sums1(a, sums(tag), (int)gridDim.x, tag, &sh.bad[1], tot);
             if ((threadIdx.x & 31) == 0) decide1(a, sh, cpub, tot);
         }
         __syncthreads();   // dU and the decision before the next constraint phase
-        if (sh.bad) return;
+        if (sh.bad[1]) return;
     }
     // every solve ends on a fresh reference: gamma = gamma_ref + gamma_lo
     // (state buffer nref & 1) and delta = 0, so dU = 0

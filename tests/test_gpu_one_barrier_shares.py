@@ -114,3 +114,27 @@ def test_recorded_step_outgrown_by_its_shares(precision):
     replay, plain = launches[2], eager[2][0].launches
     assert replay != plain
     assert launches == [plain, replay, replay, plain, replay, replay, replay, replay]
+
+
+@pytest.mark.parametrize("precision", [A.FP64, A.MIXED])
+@pytest.mark.parametrize("threads", [768, 1024])   # with and without a warp of the sums' own
+def test_waits_for_words_that_never_come_run_out(threads, precision):
+    """A block that leaves after the first grid barrier: the others' waits for its
+    velocities and sums run out, nothing moves, and the context goes on."""
+    s = system(3000)
+    with A.Context(A.params_of(s, precision=precision, tol=TOL[precision]), s.n, 12 * s.n) as ctx:
+        ctx.set_launch(threads)
+        x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+        x0, q0 = x.clone(), q.clone()
+        want = ctx.step(x, q, f)
+        moved = x.clone(), q.clone()
+        x.copy_(x0)
+        q.copy_(q0)
+        ctx.set_wait_limit(0.2)
+        ctx.inject_fault(4)
+        assert ctx.step(x, q, f, check=False).status == 4
+        assert torch.equal(x, x0) and torch.equal(q, q0)
+        ctx.set_wait_limit(5.0)
+        info = ctx.step(x, q, f)
+        assert info.solver == SOLVER_ONE and info.iters == want.iters
+        assert torch.equal(x, moved[0]) and torch.equal(q, moved[1])
