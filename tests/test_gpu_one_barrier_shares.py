@@ -1,12 +1,19 @@
-"""The one-barrier solver's launches: kernel, shared memory and what they cost."""
+"""The one-barrier solver's launches: kernel, shared memory and what they cost.
+
+Its two kernels (tagged words, and the barrier form that large systems in the
+caller's order take) and every layout of a block's share (velocities of other
+blocks' rods in rows or polled slot by slot, the step's delta and g in shared or
+global memory) sum in one order, so their solutions agree bit for bit.
+"""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
 import paper_2109_08206_gb300 as A  # noqa: E402
 
-from test_gpu_one_barrier import SOLVER_ONE, SOLVERS_TWO, system  # noqa: E402
-from test_gpu_parity import dev  # noqa: E402
+from test_gpu_one_barrier import BAR, SOLVER_ONE, SOLVERS_TWO, steps, system  # noqa: E402
+from test_gpu_parity import dev, host  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -138,3 +145,132 @@ def test_waits_for_words_that_never_come_run_out(threads, precision):
         info = ctx.step(x, q, f)
         assert info.solver == SOLVER_ONE and info.iters == want.iters
         assert torch.equal(x, moved[0]) and torch.equal(q, moved[1])
+
+
+# ------------------------------------------------------------ same bits
+def cell_order(s):
+    """The rods in the step's order: Morton order of their cells, then by id."""
+    box = np.asarray(s.box)
+    nc = np.maximum(1, np.floor(box / ((s.length + s.diameter + s.delta_c) * (1.0 + 1e-9)))).astype(int)
+    cell = np.minimum(((s.x - box * np.floor(s.x / box)) / (box / nc)).astype(int), nc - 1)
+    key = np.zeros(s.n, dtype=np.int64)
+    for bit in range(10):
+        for k in range(3):
+            key |= ((cell[:, k] >> bit) & 1) << (3 * bit + k)
+    return np.argsort(key, kind="stable")
+
+
+def layouts(pairs, n, esize, blocks):
+    """Of a launch of one block an SM (152 of them): the largest share's bytes, and for how many
+    blocks the velocities of other blocks' rods, and delta and g, find room."""
+    def up(b):
+        return (b + 15) // 16 * 16
+
+    P, Q = pairs[:, 0].astype(np.int64), pairs[:, 1].astype(np.int64)
+    row_p = np.concatenate([[0], np.cumsum(np.bincount(P, minlength=n))])
+    row_q = np.concatenate([[0], np.cumsum(np.bincount(Q, minlength=n))])
+    work = row_p + 2 * row_q + 2 * np.arange(n + 1)
+    start = [int(np.searchsorted(work, work[n] * b // blocks)) for b in range(blocks)] + [n]
+    by_q = np.argsort(Q, kind="stable")
+    need, shares = 0, []
+    for r0, r1 in zip(start, start[1:]):
+        c0, c1 = row_p[r0], row_p[r1]
+        other = by_q[row_q[r0]:row_q[r1]]
+        ghosts = other[(other < c0) | (other >= c1)]
+        far = Q[c0:c1]
+        halo = len(np.unique(np.concatenate([far[(far < r0) | (far >= r1)], P[ghosts]])))
+        nc, nr, nq, ng = c1 - c0, r1 - r0, len(other), len(ghosts)
+        nt = nc + ng
+        per_rod = np.diff(row_p[r0:r1 + 1]) + np.diff(row_q[r0:r1 + 1])
+        entries = int((4 * ((per_rod + 3) // 4)).sum())
+        need = max(need, up(4 * ((blocks + 3) // 4 * 4) * esize) + up((13 * nt + 9 * nr) * esize) +
+                   up((nt + ng + 2 * nr + 2) * 4) + up((nt + nq + nr) * 2))
+        used = up((12 * (nt + 1) + 3 * nr) * esize + 4 * nt + 2 * entries + 4 * nr + 24) + 6 * (nr + 1) * esize
+        shares.append((used, 6 * halo * esize, 2 * nc * esize))
+    room = need + need * 8 // 13
+    for kb in (164, 196):
+        most = kb * 1024 - 2048 - 1200
+        if need <= most:
+            room = min(room, most)
+            break
+    room = min(room, 230000)
+    rows = [used + h <= room for used, h, _ in shares]
+    spare = [used + (h if fits else 0) + d <= room for (used, h, d), fits in zip(shares, rows)]
+    return int(need), sum(rows), sum(spare)
+
+
+@pytest.mark.parametrize("n,precision,spills", [(17000, A.FP64, False), (17000, A.MIXED, False),
+                                                (35500, A.FP64, True), (72000, A.MIXED, True)])
+def test_barrier_form_repeats_the_tagged_form(n, precision, spills):
+    """Rods numbered in the step's order make solve_lcp (the barrier form above
+    16,000 rods) the solve of step (tagged words), with shares that hold all of
+    their data in shared memory and shares that leave delta and g to global memory
+    or poll the other blocks' velocities."""
+    s = system(n, phi=0.10)
+    order = cell_order(s)
+    tol = TOL[precision]
+    x, q, f = dev(s.x[order]), dev(s.quat[order]), dev(s.f_nc[order])
+    rows = 12 * n
+    with A.Context(A.params_of(s, precision=precision, tol=tol), n, rows) as ctx:
+        pairs = ctx.build_neighbors(x, q)
+        _, dgeom, lq = ctx.assemble_constraints(x, q, f, pairs)
+        got, lcp = ctx.solve_lcp(q, pairs, dgeom, lq)
+        _, halos, spares = layouts(host(pairs), n, 8 if precision == A.FP64 else 4, 152)
+        assert (spares < 152) == spills   # (of the float64 ones a block polls as well: halos is 151)
+        listed = torch.zeros((rows, 3), dtype=torch.int32, device="cuda")
+        want = torch.zeros(rows, dtype=torch.float64, device="cuda")
+        step = ctx.step(x, q, f, pairs_out=listed, gamma_out=want)
+    assert step.solver == lcp.solver == SOLVER_ONE
+    assert torch.equal(listed[:step.n_pairs], pairs)
+    assert (step.iters, step.residual) == (lcp.iters, lcp.residual) and lcp.residual <= tol
+    assert torch.equal(want[:step.n_pairs], got)
+
+
+# ------------------------------------------- against the two-barrier schedule
+def displacement(s, q, pairs, dgeom, g):
+    """h M D gamma of the centres, unique where gamma is not."""
+    i, j = pairs[:, 0].long(), pairs[:, 1].long()
+    F = torch.zeros((s.n, 3), dtype=torch.float64, device="cuda")
+    F.index_add_(0, i, dgeom[:, 0:3] * g[:, None])
+    F.index_add_(0, j, -dgeom[:, 0:3] * g[:, None])
+    qs = q / q.norm(dim=1, keepdim=True)
+    w, a, b, c = qs.unbind(1)
+    p = torch.stack([2 * (a * c + w * b), 2 * (b * c - w * a), w * w - a * a - b * b + c * c], 1)
+    perp = 4 * np.pi * s.viscosity * s.length / np.log(2 * s.length / s.diameter)
+    return host(s.dt / perp * (F + p * (p * F).sum(1, keepdim=True)))
+
+
+@pytest.mark.parametrize("n,precision,phi", [(16001, A.FP64, 0.06), (16001, A.MIXED, 0.06), (30000, A.FP64, 0.06),
+                                             (16000, A.FP64, 0.10), (16000, A.MIXED, 0.20)])
+def test_solve_lcp_in_caller_order(n, precision, phi):
+    """The barrier form (above 16,000 rods), and the tagged one where some blocks
+    poll the other blocks' velocities for want of room."""
+    s = system(n, phi=phi)
+    tol, bar = BAR[precision]
+    got = []
+    for barriers in (1, 2):
+        with A.Context(A.params_of(s, precision=precision, tol=tol), n, 12 * n) as ctx:
+            ctx.set_solver_schedule(barriers)
+            x, q, f = dev(s.x), dev(s.quat), dev(s.f_nc)
+            pairs = ctx.build_neighbors(x, q)
+            _, dgeom, lq = ctx.assemble_constraints(x, q, f, pairs)
+            if n <= 16000:
+                _, halos, _ = layouts(host(pairs), n, 8 if precision == A.FP64 else 4, 152)
+                assert halos < 152
+            g, info = ctx.solve_lcp(q, pairs, dgeom, lq)
+            assert info.solver == SOLVER_ONE if barriers == 1 else info.solver in SOLVERS_TWO
+            assert info.residual <= tol
+            got.append(displacement(s, q, pairs, dgeom, g))
+    if phi < 0.2:
+        assert np.abs(got[0] - got[1]).max() <= bar
+    else:   # a dense pack: forces far from unique, motion in the mean
+        assert np.linalg.norm(got[0] - got[1]) <= 1e-3 * np.linalg.norm(got[1])
+
+
+@pytest.mark.parametrize("precision", [A.FP64, A.MIXED])
+def test_two_rods_in_contact(precision):
+    """One block, one slot."""
+    s = system(2, seed=2)
+    with A.Context(A.params_of(s, precision=precision), 2, 64) as ctx:
+        assert len(ctx.build_neighbors(dev(s.x), dev(s.quat))) == 1
+    steps(s, precision, 768, 0)
