@@ -205,6 +205,18 @@ def traffic_from_profile(kernel_src: Path, shape, kernel: str):
     return float(rec["dram_bytes_per_launch"])
 
 
+def solver_kernel(solver, tn: str, shape, n: int):
+    """Name of the solver kernel behind aLENS_info.solver.  A single system's
+    steps run the one-barrier solver as k_bbpgd1, but as its barrier form with 1024
+    workers above 16,000 rods; several blocks an SM, and other shapes of more
+    than 768 workers, take the one or the other by the shares' sizes."""
+    if solver == 1 and shape is not None and (shape[0] > 768 or shape[1] > 1):
+        if shape[0] > 992 and shape[1] <= 1 and n > 16000:
+            return f"k_bbpgd1_meet<{tn}>"
+        return f"k_bbpgd1<{tn}> or k_bbpgd1_meet<{tn}>"
+    return {1: f"k_bbpgd1<{tn}>", 2: f"k_bbpgd<{tn},1>", 3: f"k_bbpgd<{tn},0>", 4: f"k_bbpgd_sys<{tn}>"}.get(solver)
+
+
 def spatial_sample(s, target):
     """Rods of the workload whose centres fall in the cube [0, a)^3, with a
     chosen so that about `target` rods fall inside; the cube is treated as a
@@ -781,8 +793,7 @@ def run_ours(args):
     achieved = alg_bytes / (ms_solve / 1e3) / 1e9
     solver = infos[-1].get("solver")
     tn = "double" if head == A.FP64 else "float"
-    kernel = {1: f"k_bbpgd1<{tn}>", 2: f"k_bbpgd<{tn},1>", 3: f"k_bbpgd<{tn},0>",
-              4: f"k_bbpgd_sys<{tn}>"}.get(solver, f"k_bbpgd<{tn}>")
+    kernel = solver_kernel(solver, tn, shape_now, n) or f"k_bbpgd<{tn}>"
     traffic = traffic_from_profile(ROOT / "paper_2109_08206_gb300" / "csrc" / "solve.cu", shape_now, kernel) \
         if args.workload == "n100k_phi010" else None   # the committed capture is of this workload
     # the whole step against the same peak: solve bytes plus the search,
@@ -817,8 +828,7 @@ def run_ours(args):
         ms64_solve = statistics.mean(i["ms_solve"] for i in inf64)
         fp64 = {"value": replica_value(ms64_step, n * spc, ws), "unit": UNIT, "ms_per_step": ms64_step,
                 "launch_shape": list(shape64),
-                "solver_kernel": {1: "k_bbpgd1<double>", 2: "k_bbpgd<double,1>", 3: "k_bbpgd<double,0>",
-                                  4: "k_bbpgd_sys<double>"}.get(inf64[-1].get("solver")),
+                "solver_kernel": solver_kernel(inf64[-1].get("solver"), "double", shape64, n),
                 "roofline_frac": statistics.mean(sb64) / (ms64_solve / 1e3) / 1e9 / peak,
                 "step_frac": None if isinstance(job, GradJob) else
                 (statistics.mean(sb64) + spc * step_other_bytes(n, inf64[-1]["n_pairs"], 8))

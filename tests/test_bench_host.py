@@ -82,3 +82,11 @@ def test_sibling_jobs_draw_other_inputs_of_the_same_class():
     a, b = bench.make_job("n1000_box40"), bench.make_job("n1000_box40", sibling=True)
     assert a.n == b.n and a.s.box == b.s.box and a.s.tol == b.s.tol
     assert not np.array_equal(a.s.x, b.s.x)
+
+
+def test_solver_kernel_names_the_barrier_form():
+    assert bench.solver_kernel(1, "float", (768, 1), 100_000) == "k_bbpgd1<float>"
+    assert bench.solver_kernel(1, "float", (1024, 1), 100_000) == "k_bbpgd1_meet<float>"
+    assert "k_bbpgd1_meet<double>" in bench.solver_kernel(1, "double", (512, 2), 20_000)
+    assert bench.solver_kernel(3, "double", (1024, 1), 100_000) == "k_bbpgd<double,0>"
+    assert bench.solver_kernel(4, "float", (1024, 8), 100_000) == "k_bbpgd_sys<float>"
