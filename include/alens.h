@@ -325,10 +325,12 @@ ALENS_API aLENS_status aLENS_set_batch_graph(aLENS_ctx* ctx, int32_t enable);
  * schedule) runs without a graph; if that step ran the one-barrier solver
  * (aLENS_info.solver = 1), the second call records the step and runs it,
  * and later calls replay it.  In the recorded step the solver is launched
- * with the whole shared-memory budget of its launch shape and checks on the
+ * with shared memory for the shares of the step before it and checks on the
  * device that every block's share fits; when one does not (the pairs moved
  * into a denser arrangement), nothing moves and the call runs the step
- * without a graph, as do all later calls with that key.  Kernels sized by
+ * without a graph, and the next call records it anew.  A key whose shares
+ * outgrow all the shared memory of the launch shape stays without a graph.
+ * Kernels sized by
  * the constraint count are launched for the context's capacity and read the
  * count on the device; a step whose pairs exceed the capacity changes
  * nothing and returns ALENS_ERR_CAPACITY with the required count.  Steps

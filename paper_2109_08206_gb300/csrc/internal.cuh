@@ -357,8 +357,10 @@ struct aLENS_ctx {
     void* solve_ws;          // typed solver buffers (sized for double)
     alens::SolveBufs<double> sb64;
     alens::SolveBufs<float> sb32;
-    double* partials;        // [max_blocks + 4][8]: [4][nb] block sums
-    uint4* xch;              // one-barrier solver's tagged words: 2 velocity buffers (at most 4 words a rod), block sums
+    double* partials;        // [max_blocks + 4][8]: [4][nb] block sums ([2][4][nb], nb rounded up to 4, in the barrier
+                             // form of the one-barrier solver)
+    uint4* xch;              // one-barrier solver's tagged words: 2 velocity buffers (at most 4 words a rod), block sums;
+                             // its barrier form's second velocity buffer [n][6]
     int max_blocks;
     int* bstart;             // [max_blocks + 1] solver block boundaries (rod ranks)
     unsigned* bar;           // [4]
@@ -405,7 +407,8 @@ struct aLENS_ctx {
     cudaEvent_t ev_fork, ev_join;  // side waits for ev_fork; the step's stream for ev_join
     int graph_launches;      // kernels in the graph
     int graph_state;         // 0 nothing, 1 the key below ran eagerly once, 2 a graph of it is instantiated,
-                             // 3 the key stays eager (its solver reads back, or a recorded step redid)
+                             // 3 the key stays eager (its solver reads back, or a recorded step with all the
+                             // shared memory there is redid)
     struct GraphKey {
         int64_t n;
         const void* ptr[6];  // x, quat, f_nc, pairs_out, gamma_out, vel_out

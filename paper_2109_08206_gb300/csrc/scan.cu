@@ -1,8 +1,7 @@
 // Exclusive prefix sums of int32 counts (CSR row pointers, cell starts), one
 // array or two of the same length at once (grid.y), and the zeroing of count
 // arrays.  Small steps are bound by their launches (about 3 us each, most of
-// it the launch): a single-system step
-// had 11 memsets and 30 kernels.
+// it the launch), so each of these is one where it can be.
 // Up to kScanSmall entries one block scans an array tile after tile (1.6e4
 // entries: 4 us; two launches 6 to 9).  More: per-tile totals, then per-tile
 // scans, each block adding the totals of the tiles before it (a few thousand at

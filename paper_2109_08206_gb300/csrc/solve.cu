@@ -1372,8 +1372,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd(SolveArgs<T> a)
 // ms a step, 5e3 rods 0.86 -> 0.66, 2e4 rods 1.98 -> 1.45, 5e4 rods 1.43 ->
 // 1.25, 1e5 rods 3.90 -> 3.60 (366 iterations), 1e4 rods float64 2.17 -> 1.56.
 // Where the rods come in no spatial order (a large solve_lcp) nearly every
-// slot's other end is in the halo and the polls cost more than they save: those
-// keep the barrier (k_bbpgd1_meet).
+// slot's other end is in the halo and the polls cost more than they save, and
+// where a launch leaves no L1 for what this kernel spills: those keep the
+// barrier (k_bbpgd1_meet, variant1).
 
 // A block's share: rods [r0, r1), owned constraints [c0, c1) in slots
 // [0, nc), ghosts in slots [nc, nt).
@@ -2328,7 +2329,9 @@ __device__ __forceinline__ void decide1(const SolveArgs<T>& a, Shared1<T>& sh, i
 }
 
 // MAXT: the most threads of a launch (kThreads1: the default shape and its
-// further warp, with 72 registers a thread; 1024: every other shape).
+// further warp, with 72 registers a thread; 1024: every other shape, with 64).
+// Neither holds all it needs: a thread spills 444 bytes (float64; 392 read
+// back) or 92 (float32; 252) in the first and 576 or 204 in the second.
 constexpr int kThreads1 = 800;
 template <typename T, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ SolveArgs<T> a)
@@ -2515,14 +2518,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_bbpgd1(const __grid_constant__ Solv
 }
 
 // ---------------------------------------------------------------------
-// The same iteration with one grid barrier, for large systems whose rods come
-// in no spatial order (solve_lcp takes the caller's order): nearly every
-// slot's other end then lies in another block, and the halo of tagged words
-// costs more to poll than a barrier and plain gathers of the slots' own words
-// (solve, barrier / tagged: 3e4 rods 0.65 / 0.84 ms, 5e4 rods 2.10 / 2.48;
-// 8e3 rods 0.71 / 0.56, so the line lies between).  One thread per rod, a
-// slot's values in columns; the sums are the same in the same order, and so
-// is every bit.
+// The same iteration with one grid barrier and without spills, for the
+// launches that variant1 names and for large systems whose rods come in no
+// spatial order (solve_lcp takes the caller's order): nearly every slot's
+// other end then lies in another block, and the halo of tagged words costs more
+// to poll than a barrier and plain gathers of the slots' own words (solve, ms,
+// barrier / tagged: mixed 8e3 rods 0.70 / 0.56, 1.6e4 0.99 / 0.85, 2e4 1.11 /
+// 0.96, 5e4 2.76 / 3.03; float64 1.6e4 5.64 / 4.87, 2e4 5.45 / 4.48: the line
+// lies below the crossing).  One thread per rod, a slot's values in columns;
+// the sums are the same in the same order, and so is every bit
+// (test_barrier_form_repeats_the_tagged_form).
 constexpr int kMeetRods = 16000;
 namespace meet {
 
@@ -3043,9 +3048,6 @@ __device__ __forceinline__ void warps_totals(const Own1<T>& o, int nb, T* tot)
     asm volatile("bar.sync 1, 128;\n" ::: "memory");
 }
 
-// Loop states: what the last constraint phase was (its sums are what the
-// last barrier published), and the decision taken for the next rod phase.
-
 template <typename T>
 __global__ void __launch_bounds__(1024, 1) k_bbpgd1_meet(SolveArgs<T> a)
 {
@@ -3226,7 +3228,7 @@ __global__ void __launch_bounds__(1024, 1) k_bbpgd1_meet(SolveArgs<T> a)
 }  // namespace meet
 
 // The work-balanced split and what its shares need, one thread block per solver block b
-// in one launch (three before): the share's two boundaries (bstart; a warp
+// in one launch: the share's two boundaries (bstart; a warp
 // each), the two-barrier kernel's largest shared-memory share and rod count
 // over the blocks (need, maxrods), and the one-barrier kernel's (need1; ghosts
 // counted from the block's other-side entries; a share whose slot or rod
@@ -3577,7 +3579,7 @@ static long long dyn_within(int kb, int blocks)
 //    every block's sums, and the halo grows with the blocks (1.0e4 rods at 512 x
 //    2 and 256 x 4 0.91 / 0.91 and 0.88 / 0.87, 1.2e4 1.18 / 1.18 and 1.02 /
 //    1.04, 3e4 1.44 / 1.47 and 1.93 / 2.45).
-// Without it elsewhere, with 80 registers a thread in the default shape.
+// Without it elsewhere, in the default shape with 72 registers a thread.
 enum { V_MEET = 0, V_WIDE = 1, V_ANY = 2 };
 constexpr int kMeetRodsSeveral = 10000;
 template <typename T>
@@ -3630,12 +3632,14 @@ static cudaError_t ready1(aLENS_ctx* ctx, int variant, size_t budget, int& threa
 // the share itself leaves, up to 92 KB of it: the kernel's spilled registers
 // live there, and where the largest division leaves 28 KB they go to L2 (the
 // steps of the division are the device's).  Solve, ms, with the whole room
-// and so: 3e4 rods float64 7.86 / 5.20, 1.6e4 rods float64 in caller order
-// 8.22 / 4.87, 3e4 rods float64 at 512 x 2 11.5 / 8.45, 6e4 rods mixed 2.14 /
-// 1.91; a halo that finds no room then is polled slot by slot.
+// and so: 3e4 rods float64 7.86 / 5.21, 1.6e4 rods float64 in caller order
+// 8.16 / 4.85, 2e4 rods float64 at 512 x 2 6.23 / 4.97, 6e4 rods mixed 2.18 /
+// 1.88; a halo that finds no room then is polled slot by slot.
 // The driver divides an SM for as many blocks as their registers allow
 // (by_regs), so a launch of fewer asks for little enough that all those fit
-// the division, or for too much for one more than bps.
+// the division, or for too much for one more than bps (2e4 rods float64 at 256
+// x 3 7.28 / 5.62).  Naming the division at the launch instead does not do: it
+// can hold fewer blocks than the cooperative grid needs on the SM.
 template <typename T>
 static long long request1(const aLENS_ctx* ctx, int by_regs, long long need, long long budget)
 {
